@@ -181,7 +181,8 @@ typedef struct {
                            launched merge's operands read and result written once (complex64) */
   int32_t n_fused;      /* dense 4x4 blocks (precontracted runs of gates on two qubits) in the forward passes;
                            TN_PLAN_BLOCKS: the 2^k x 2^k blocks (n_passes = GEMM launches = blocks - 1) */
-  int32_t reserved_stats;
+  int32_t q428_launches;  /* TN_PLAN_Q428: kernel launches per call (n_passes counts the gates, hbm_bytes a
+                             gate-by-gate contraction's bytes); 0 for other plans */
 } tn_plan_stats;
 
 /* Pauli sum H = sum_t coef[t] * P_t (host memory, read during tn_build_observable only).

@@ -283,9 +283,16 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
   p->K = K;
   std::string err;
   if (o.flags & TN_PLAN_Q428) {
-    p->q428 = new std::vector<Q428Gate>();
-    q428_build(*c, *p->q428);
-    if (!p->host_only) TN_CUDA(cudaGetDevice(&p->device), "cudaGetDevice");
+    p->q428 = q428_build(*c);
+    if (!p->host_only) {
+      cudaError_t e = cudaGetDevice(&p->device);
+      if (e == cudaSuccess) e = q428_upload(p->q428);
+      if (e != cudaSuccess) {
+        q428_free(p->q428);
+        delete p;
+        return cuda_fail(e, "fixed-point plan tables");
+      }
+    }
     p->ws_bytes = 0;
     *out = p;
     return TN_OK;
@@ -507,9 +514,10 @@ tn_status tn_plan_get_stats(const tn_plan *p, tn_plan_stats *st) {
   st->n_phases = (int)p->fwd.phases.size();
   st->n_ops = (long long)p->fwd.ops.size();
   st->n_fused = p->n_fused;
-  if (p->q428) {  // one launch per gate, each reading and writing every amplitude (int32 pairs)
-    st->n_passes = (int)p->q428->size();
-    st->hbm_bytes = 8.0 * std::ldexp(1.0, p->n) * (1.0 + 2.0 * (double)p->q428->size());
+  if (p->q428) {  // gate by gate: each reads and writes every amplitude (int32 pairs); launches hold many gates
+    st->n_passes = q428_gates(p->q428);
+    st->hbm_bytes = 8.0 * std::ldexp(1.0, p->n) * (1.0 + 2.0 * (double)q428_gates(p->q428));
+    st->q428_launches = q428_launches(p->q428);
     return TN_OK;
   }
   st->tile_qubits = p->T;
@@ -552,7 +560,7 @@ tn_status tn_plan_get_stats(const tn_plan *p, tn_plan_stats *st) {
 
 void tn_free_plan(tn_plan *p) {
   if (!p) return;
-  delete p->q428;
+  q428_free(p->q428);
   p->q428 = nullptr;
   if (p->blocks) {
     if (!p->host_only) free_blocks(*p->blocks);
@@ -760,7 +768,7 @@ tn_status tn_contract_state_q428(const tn_plan *p, int32_t *state_dev, tn_stream
   TN_CHECK_ARG(((uintptr_t)state_dev & 7) == 0, "state_dev must be 8-byte aligned");
   tn_status st = check_device(p->device);
   if (st != TN_OK) return st;
-  TN_CUDA(launch_q428(*p->q428, p->n, p->init, state_dev, reinterpret_cast<cudaStream_t>(s)), "fixed-point kernels");
+  TN_CUDA(launch_q428(p->q428, p->n, p->init, state_dev, reinterpret_cast<cudaStream_t>(s)), "fixed-point kernels");
   return TN_OK;
 }
 

@@ -431,6 +431,7 @@ struct Q428Gate {
   int pos[2];
   int32_t u[32];
 };
+struct Q428Plan;
 }  // namespace tnq
 
 namespace tnq {
@@ -440,7 +441,7 @@ struct BlockPlan;
 struct tn_plan {
   tnq::NetPlan *net = nullptr;  // TN_PLAN_NETWORK plans: pairwise network contraction
   tnq::BlockPlan *blocks = nullptr;  // TN_PLAN_BLOCKS plans: uniform square blocks
-  std::vector<tnq::Q428Gate> *q428 = nullptr;  // TN_PLAN_Q428 plans: quantised gate list
+  tnq::Q428Plan *q428 = nullptr;  // TN_PLAN_Q428 plans: quantised gates, passes and phases
   int n;
   long long n_gates;
   int batch;

@@ -57,7 +57,7 @@ class TnPlanStats(C.Structure):
                 ("net_merges", C.c_int32), ("net_max_log2", C.c_int32), ("net_tensor_merges", C.c_int32),
                 ("net_folded_merges", C.c_int32), ("bwd_flops", C.c_double),
                 ("net_sliced", C.c_int32), ("net_batch_log2", C.c_int32), ("net_cost", C.c_double),
-                ("net_bytes", C.c_double), ("n_fused", C.c_int32), ("reserved_stats", C.c_int32)]
+                ("net_bytes", C.c_double), ("n_fused", C.c_int32), ("q428_launches", C.c_int32)]
 
 
 class TnTuneOpts(C.Structure):

@@ -126,3 +126,70 @@ def test_30_qubits_closed_form():
     bits = (pre[:, None] >> (n - 1 - np.arange(n))[None, :]) & 1
     sign = 1 - 2 * (np.sum(bits[:, :-1] * bits[:, 1:], axis=1) & 1)
     assert np.array_equal(got, sign * a)
+
+
+def _exact_ints(circ):
+    """The circuit in Q4.28 with Python integers: any entries, any amplitudes (the oracle's int64 sums
+    stop at 2^29), saturating after every gate."""
+    from oracle import fixedpoint as F
+    from oracle.statevector import gate_matrix
+    n = circ.n_qubits
+    lo, hi = F.INT32_MIN, F.INT32_MAX
+    st = [(0, 0)] * (1 << n)
+    st[circ.init_basis] = (1 << 28, 0)
+
+    def rnd(v):
+        return min(max((v + (1 << 27)) >> 28, lo), hi)
+    for g in circ.gates:
+        ur, ui = (m.tolist() for m in F.quantize_matrix(gate_matrix(circ, g, None)))
+        bits = [n - 1 - q for q in g.qubits]
+        d = 1 << len(bits)
+        out = list(st)
+        for x in range(1 << n):
+            if any((x >> b) & 1 for b in bits):
+                continue
+            idx = [x | sum(((k >> (len(bits) - 1 - i)) & 1) << b for i, b in enumerate(bits)) for k in range(d)]
+            v = [st[i] for i in idx]
+            for r in range(d):
+                out[idx[r]] = (rnd(sum(ur[r][k] * v[k][0] - ui[r][k] * v[k][1] for k in range(d))),
+                               rnd(sum(ur[r][k] * v[k][1] + ui[r][k] * v[k][0] for k in range(d))))
+        st = out
+    a = np.array(st, dtype=np.int64)
+    return a[:, 0], a[:, 1]
+
+
+@pytest.mark.parametrize("n", [3, 4, 5, 8])
+def test_large_amplitudes_and_entries_saturate(n):
+    """Gates that grow the state past 2^29, into saturation, and entries at the int32 limits: the forms
+    that may not assume small amplitudes, and sign flips and exchanges of saturated values."""
+    rng = np.random.default_rng(900 + n)
+    gates = [C.Gate("H", (q,)) for q in range(n)]
+    for _ in range(10):
+        q, r = (int(v) for v in rng.choice(n, size=2, replace=False))
+        m = tuple(complex(a, b) for a, b in rng.uniform(-1.6, 1.6, size=(4, 2)))
+        gates += [C.Gate("MAT1", (q,), (), -1, m), C.Gate("CZ", (q, r)), C.Gate("RX", (r,), (1.1,)),
+                  C.Gate("CNOT", (r, q)), C.Gate("U3", (q,), (0.4, 1.3, 2.2)), C.Gate("T", (r,)), C.Gate("Z", (q,))]
+    gates.append(C.Gate("MAT1", (0,), (), -1, (-9.0 + 0j, 0j, 1j, 9.0 + 0j)))      # INT_MIN and INT_MAX entries
+    gates.append(C.Gate("MAT1", (1,), (), -1, (-9.0 + 0j, 0.3j, 1j, 2.5 - 9.0j)))
+    gates.append(C.Gate("MAT1", (2,), (), -1, (1.0 + 0j, 0j, 0j, -9.0j)))          # diagonal
+    gates += [C.Gate("CZ", (0, 1)), C.Gate("CZ", (0, 1)), C.Gate("CZ", (1, 2)), C.Gate("SWAP", (0, 2))]
+    c = C.Circuit(n, gates)
+    re, im = _q428(c)
+    rr, ri = _exact_ints(c)
+    assert max(abs(rr).max(), abs(ri).max()) >= (1 << 31) - 1  # the case saturates
+    assert np.array_equal(re, rr) and np.array_equal(im, ri)
+
+
+def test_pass_records_at_their_limits():
+    """More ops, matrix entries and phases than one pass stages: runs of dense 4x4s on changing pairs
+    (2048 entries hold 64 of them), of one-qubit gates on one qubit (128 ops) and on five (64 phases)."""
+    rng = np.random.default_rng(31)
+    n = 9
+    gates = []
+    for _ in range(70):
+        a, b = (int(v) for v in rng.choice(n, size=2, replace=False))
+        q = np.linalg.qr(rng.normal(size=(4, 4)) + 1j * rng.normal(size=(4, 4)))[0]
+        gates.append(C.Gate("MAT2", (a, b), (), -1, tuple(complex(z) for z in q.reshape(-1))))
+    gates += [C.Gate("U3", (3,), tuple(rng.uniform(0, 6, 3))) for _ in range(131)]
+    gates += [C.Gate("U3", (int(4 * k % 9),), tuple(rng.uniform(0, 6, 3))) for k in range(300)]
+    _assert_bit_exact(C.Circuit(n, gates, init_basis=300))
