@@ -678,6 +678,7 @@ tn_status tn_build_observable(int32_t n_qubits, const tn_pauli_sum *H, tn_observ
       --left;
     }
     o->passes.push_back(make_pass(S, tb, (int)o->terms.size()));
+    o->passes.back().n_diag = first ? (int)diag.size() : 0;
     first = false;
   }
   if ((int)o->passes.size() > kMaxRedPasses) {

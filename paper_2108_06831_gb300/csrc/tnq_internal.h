@@ -495,6 +495,8 @@ static_assert(sizeof(DevTerm) == 32, "DevTerm layout");
 struct alignas(16) RedPass {
   int32_t T, n_outer;
   int32_t term_begin, term_end;
+  int32_t n_diag;  // the first n_diag of the pass's terms flip nothing (xl = 0), the others do
+  int32_t pad;
   uint8_t tile_pos[16];
   uint8_t outer_pos[40];
 };

@@ -153,3 +153,47 @@ def test_autograd_function():
     for b, w in ((0, 1.0), (1, -2.0)):
         gref = w * GR.param_shift_grad(c, H, params[b])
         assert np.linalg.norm(g[b] - gref) / max(np.linalg.norm(gref), 1e-3) <= 1e-4
+
+
+def _mixed_sum(n, n_terms, seed):
+    """Random Pauli strings: dense ones up to 10 qubits, on three qubits beyond (their flips fit a tile);
+    several terms share their flips, some have none."""
+    rng = np.random.default_rng(seed)
+    H = C.PauliSum(n)
+    for k in range(n_terms):
+        if n <= 10:
+            s = "".join("IXYZ"[int(v)] for v in rng.integers(0, 4, size=n))
+            H.coef.append(float(rng.normal()))
+            H.strings.append(s)
+            if k % 4 == 0:  # the same flips with other signs, and a Z string
+                H.coef.append(float(rng.normal()))
+                H.strings.append(s.translate(str.maketrans("XYIZ", "YXZI")))
+                H.coef.append(float(rng.normal()))
+                H.strings.append(s.translate(str.maketrans("XY", "ZI")))
+        else:
+            qs = rng.choice(n, size=3, replace=False)
+            for ops in ("XYZ", "YXZ", "XXI", "YYI", "ZZZ", "IIY"):
+                H.add(float(rng.normal()), [(int(q), p) for q, p in zip(qs, ops) if p != "I"])
+    return H
+
+
+@pytest.mark.parametrize("n", [1, 2, 4, 7, 8, 9, 10, 11, 12, 13, 16])
+def test_pauli_sums_over_tile_sizes(n):
+    """Tiles of every size (one row of fewer than 256 amplitudes up to 16 rows), flips on thread bits and
+    on row bits, Z masks on both and outside the tile: the direct energy and the one summed from H psi,
+    within the stated FP32 bound (terms + 16) 2^-24 sum |c| plus the state's own FP32 error."""
+    from oracle import observables as OB
+    tn = _tn()
+    c = C.hea(n, 2)
+    H = _mixed_sum(n, 12, 300 + n)
+    batch = 2
+    params = C.hea_params(c.n_params, batch, 20 + n)
+    ctr = tn.Contractor(c, target=tn.TARGET_EXPECTATION, batch=batch)
+    obs = tn.Observable(H)
+    e, _ = ctr.expectation_value_and_grad(obs, _dev(params))
+    direct = ctr.expectation(obs, _dev(params)).cpu().numpy()
+    bound = (len(H.coef) + 16 + len(c.gates)) * 2.0 ** -24 * float(np.abs(H.coef).sum())
+    for b in range(batch):
+        ref = OB.expectation(c, H, params[b])
+        assert abs(direct[b] - ref) <= bound
+        assert abs(e[b].item() - ref) <= bound
