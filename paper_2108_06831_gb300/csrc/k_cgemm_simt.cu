@@ -27,8 +27,8 @@ constexpr int kThreads = 256;
 struct StagedMap {
   OutMap map;
   int lgn, L, nlo, pairs;
-  int s_lo[64], s_hi[64];       // staging offsets (complex)
-  long long g_lo[64], g_hi[64];  // stored offsets (complex)
+  int s_lo[64], s_hi[128];       // staging offsets (complex)
+  long long g_lo[64], g_hi[128];  // stored offsets (complex)
 };
 void build_staged(StagedMap &sm, const OutMap &om, long long M, long long N, int BM, int BN);
 
@@ -47,6 +47,39 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Permuted output: the tile staged in shared memory (smem, written by the caller, not yet synchronised)
+// goes back in stored-index order, u -> (staging offset, stored offset) from the host-built tables
+// (copied to shared memory: lanes index them divergently).
+template <int THREADS>
+__device__ __forceinline__ void store_staged(const float2 *smem, float2 *__restrict__ C, long long gbase,
+                                             const StagedMap &om) {
+  __shared__ int s_lo[64], s_hi[128];
+  __shared__ long long g_lo[64], g_hi[128];
+  const int L = om.L, nlo = om.nlo, lo_mask = (1 << om.nlo) - 1;
+  if (threadIdx.x < 64) {
+    s_lo[threadIdx.x] = om.s_lo[threadIdx.x];
+    g_lo[threadIdx.x] = om.g_lo[threadIdx.x];
+  }
+  const int hi = THREADS - 1 - (int)threadIdx.x;  // the other end of the CTA
+  if (hi < 1 << (L - nlo)) {
+    s_hi[hi] = om.s_hi[hi];
+    g_hi[hi] = om.g_hi[hi];
+  }
+  __syncthreads();
+  if (L == 0) {
+    if (threadIdx.x == 0) C[gbase] = smem[0];
+  } else if (om.pairs) {  // u, u + 1 adjacent in memory: 16-byte stores
+    for (int u = 2 * threadIdx.x; u < (1 << L); u += 2 * THREADS) {
+      const float2 x0 = smem[s_lo[u & lo_mask] + s_hi[u >> nlo]];
+      const float2 x1 = smem[s_lo[(u + 1) & lo_mask] + s_hi[(u + 1) >> nlo]];
+      *reinterpret_cast<float4 *>(C + gbase + g_lo[u & lo_mask] + g_hi[u >> nlo]) = make_float4(x0.x, x0.y, x1.x, x1.y);
+    }
+  } else {
+    for (int u = threadIdx.x; u < (1 << L); u += THREADS)
+      C[gbase + g_lo[u & lo_mask] + g_hi[u >> nlo]] = smem[s_lo[u & lo_mask] + s_hi[u >> nlo]];
+  }
+}
 
 template <int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__(kThreads, 2) k_cgemm_fp32(long long M, long long N, long long K, long long k_len,
@@ -137,38 +170,131 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_fp32(long long M, long lo
         if (gm < M && gn < N) Ob[gm * N + gn] = acc[i][j];
       }
   } else {
-    // Permuted output: the tile is staged in shared memory and written back in stored-index
-    // order, u -> (staging offset, stored offset) from the host-built tables (copied to shared
-    // memory: lanes index them divergently).
-    __shared__ int s_lo[64], s_hi[64];
-    __shared__ long long g_lo[64], g_hi[64];
-    if (threadIdx.x < 64) {
-      s_lo[threadIdx.x] = om.s_lo[threadIdx.x];
-      g_lo[threadIdx.x] = om.g_lo[threadIdx.x];
-    } else if (threadIdx.x < 128) {
-      s_hi[threadIdx.x - 64] = om.s_hi[threadIdx.x - 64];
-      g_hi[threadIdx.x - 64] = om.g_hi[threadIdx.x - 64];
-    }
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
       for (int j = 0; j < TN; ++j) smem[(ty + (BM / TM) * i) * (BN + 1) + tx + NX * j] = acc[i][j];
-    __syncthreads();
-    const long long gbase = map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0);
-    const int L = om.L, nlo = om.nlo, lo_mask = (1 << om.nlo) - 1;
-    if (L == 0) {
-      if (threadIdx.x == 0) C[gbase] = smem[0];
-    } else if (om.pairs) {  // u, u + 1 adjacent in memory: 16-byte stores
-      for (int u = 2 * threadIdx.x; u < (1 << L); u += 2 * kThreads) {
-        const float2 x0 = smem[s_lo[u & lo_mask] + s_hi[u >> nlo]];
-        const float2 x1 = smem[s_lo[(u + 1) & lo_mask] + s_hi[(u + 1) >> nlo]];
-        *reinterpret_cast<float4 *>(C + gbase + g_lo[u & lo_mask] + g_hi[u >> nlo]) =
-            make_float4(x0.x, x0.y, x1.x, x1.y);
-      }
-    } else {
-      for (int u = threadIdx.x; u < (1 << L); u += kThreads)
-        C[gbase + g_lo[u & lo_mask] + g_hi[u >> nlo]] = smem[s_lo[u & lo_mask] + s_hi[u >> nlo]];
+    store_staged<kThreads>(smem, C, map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0), om);
+  }
+}
+
+// The wide form, for outputs of more than 32 columns with enough tiles to fill the SMs: 128 x 64 tiles,
+// 128 threads of 8 x 8 complex accumulators.  What bounds the 64 x 64 form (4 x 4 accumulators) is
+// shared memory: each step of K reads TM + TN elements per thread for TM TN complex multiply-adds, 16
+// clocks of a warp's loads per 16 clocks of its FMAs; 8 x 8 reads half as much.  Bound now: FMA issue
+// (78% of issue slots).  4096^3: 11.9 -> 9.6 ms (46 -> 57.5 TFLOP/s); batch 64, 4096 x 64 x 64: 204 ->
+// 168 us.  The packed FP32x2 multiply-adds are slower here (39.5 against 57.9 TFLOP/s at 2432 x 2048 x
+// 512): every operand of the complex product has to be duplicated or swapped into a register pair, and
+// those moves take the FMA pipe's slots.  Same roundings in the same order as the 64 x 64 form.
+// Slices of 16 K are staged by cp.async, three in flight, in rows of 18 elements (16-byte aligned, a
+// warp's reads conflict-free); VEC: 16-byte copies, for even K.  Four steps of K are unrolled (2, 8 and
+// 16 measured 9.8, 9.8 and 10.3 ms).
+constexpr int kWideThreads = 128, kWideK = 16, kWideStages = 3;
+constexpr int kWideLd = kWideK + 2;
+template <int BM, int BN>
+constexpr size_t wide_smem() {
+  constexpr int slices = kWideStages * (BM + BN) * kWideLd, tile = BM * (BN + 1);
+  return sizeof(float2) * (slices > tile ? slices : tile);
+}
+
+// asynchronous copy of the first n of BYTES bytes, the rest zeros
+template <int BYTES>
+__device__ __forceinline__ void cp_async_z(void *dst, const void *src, int n) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(BYTES), "r"(n)
+               : "memory");
+}
+
+template <bool VEC, int BM, int BN, int TM, int TN, int MINB>
+__global__ void __launch_bounds__(kWideThreads, MINB) k_cgemm_fp32_wide(long long M, long long N, long long K,
+                                                                     const float2 *__restrict__ A,
+                                                                     const float2 *__restrict__ B,
+                                                                     float2 *__restrict__ C,
+                                                                     const __grid_constant__ StagedMap om) {
+  static_assert((BM / TM) * (BN / TN) == kWideThreads, "one thread per TM x TN block");
+  constexpr int NX = BN / TN, NY = BM / TM, kSlice = (BM + BN) * kWideLd;
+  extern __shared__ __align__(16) float2 smem_w[];
+  pdl_wait();
+  pdl_trigger();
+  const long long tiles_n = (N + BN - 1) / BN;
+  const long long b = blockIdx.z;
+  const long long m0 = ((long long)blockIdx.x / tiles_n) * BM, n0 = ((long long)blockIdx.x % tiles_n) * BN;
+  const float2 *Ab = A + (b * M + m0) * K, *Bb = B + (b * N + n0) * K;
+  constexpr int kPer = VEC ? 2 : 1;                       // elements per copy
+  constexpr int kCols = kWideK / kPer;                    // copies per row
+  constexpr int kStep = kWideThreads / kCols;             // rows copied at once
+  const int lr = threadIdx.x / kCols, lc = (threadIdx.x % kCols) * kPer;
+  const int rows_a = (int)(M - m0 < BM ? M - m0 : BM), rows_b = (int)(N - n0 < BN ? N - n0 : BN);
+  auto load_slice = [&](int sb, long long k0) {
+    float2 *as = smem_w + sb * kSlice, *bs = as + BM * kWideLd;
+    const bool in_k = k0 + lc < K;
+    const float2 *ga = Ab + k0 + lc, *gb = Bb + k0 + lc;
+#pragma unroll
+    for (int r = lr; r < BM; r += kStep) {
+      const bool ok = in_k && r < rows_a;
+      cp_async_z<8 * kPer>(as + r * kWideLd + lc, ok ? ga + r * K : A, ok ? 8 * kPer : 0);
     }
+#pragma unroll
+    for (int r = lr; r < BN; r += kStep) {
+      const bool ok = in_k && r < rows_b;
+      cp_async_z<8 * kPer>(bs + r * kWideLd + lc, ok ? gb + r * K : B, ok ? 8 * kPer : 0);
+    }
+  };
+  const int tx = threadIdx.x % NX, ty = threadIdx.x / NX;
+  float2 acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  const int slices = (int)((K + kWideK - 1) / kWideK);
+#pragma unroll
+  for (int t = 0; t < kWideStages - 1; ++t) {
+    if (t < slices) load_slice(t, (long long)t * kWideK);
+    cp_async_commit();
+  }
+  for (int t = 0; t < slices; ++t) {
+    cp_async_wait<kWideStages - 2>();
+    __syncthreads();  // slice t has landed, and its successor's buffer (slice t - 1) is read out
+    if (t + kWideStages - 1 < slices) load_slice((t + kWideStages - 1) % kWideStages, (long long)(t + kWideStages - 1) * kWideK);
+    cp_async_commit();
+    const float2 *as = smem_w + (t % kWideStages) * kSlice + ty * kWideLd;
+    const float2 *bs = smem_w + (t % kWideStages) * kSlice + (BM + tx) * kWideLd;
+    const int left = (int)(K - (long long)t * kWideK), quads = left >= kWideK ? kWideK / 4 : (left + 3) / 4;
+#pragma unroll 1
+    for (int q = 0; q < quads; ++q, as += 4, bs += 4)
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      float2 bb[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) bb[j] = bs[NX * j * kWideLd + kk];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float2 a = as[NY * i * kWideLd + kk];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          acc[i][j].x = fmaf(a.x, bb[j].x, acc[i][j].x);
+          acc[i][j].y = fmaf(a.x, bb[j].y, acc[i][j].y);
+          acc[i][j].x = fmaf(-a.y, bb[j].y, acc[i][j].x);
+          acc[i][j].y = fmaf(a.y, bb[j].x, acc[i][j].y);
+        }
+      }
+    }
+  }
+  if (om.map.identity) {
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const long long gm = m0 + ty + NY * i, gn = n0 + tx + NX * j;
+        if (gm < M && gn < N) C[(b * M + gm) * N + gn] = acc[i][j];
+      }
+  } else {
+    __syncthreads();  // the last slice is read out; nothing is in flight
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) smem_w[(ty + NY * i) * (BN + 1) + tx + NX * j] = acc[i][j];
+    store_staged<kWideThreads>(smem_w, C, map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0), om);
   }
 }
 
@@ -335,6 +461,36 @@ cudaError_t launch_shape(long long batch, long long M, long long N, long long K,
                     (const float2 *)P, splits, total, C, om);
 }
 
+// Whether the 128 x 64 form is the faster one: both it and the 64 x 64 form run two CTAs per SM, a full
+// wave of the 64 x 64 form (half the outputs) takes 0.63 of a full wave of the wide form (46 against 58
+// TFLOP/s at 4096^3), and a last wave of at most one CTA per SM about 0.6 of a full one.  Taken when that
+// estimate gains a tenth: 1500 x 1500 x 100 54.6 -> 39.5 us; below it, for instance at 40 x 200 x 200 x
+// 200, the wide form was slower (117 against 137 us).
+bool wide_ok(long long batch, long long M, long long N) {
+  const long long slots = 2ll * num_sms();
+  auto waves = [&](long long bm, long long bn) {
+    const long long tiles = batch * ((M + bm - 1) / bm) * ((N + bn - 1) / bn), r = tiles % slots;
+    return (double)(tiles / slots) + (r == 0 ? 0.0 : 2 * r <= slots ? 0.6 : 1.0);
+  };
+  return M > 64 && waves(128, 64) < 0.9 * 0.63 * waves(64, 64);
+}
+template <int BM, int BN, int TM, int TN, int MINB>
+cudaError_t launch_wide(long long batch, long long M, long long N, long long K, const float2 *A, const float2 *B,
+                        float2 *C, const OutMap &om, cudaStream_t s) {
+  const long long tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
+  if (tiles > 0x7fffffffll || K > (1ll << 30)) return cudaErrorNotSupported;
+  StagedMap sm;
+  std::memset(&sm, 0, sizeof(sm));
+  sm.map = om;
+  if (!om.identity) build_staged(sm, om, M, N, BM, BN);
+  const bool vec = K % 2 == 0 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
+  auto *fn = vec ? k_cgemm_fp32_wide<true, BM, BN, TM, TN, MINB> : k_cgemm_fp32_wide<false, BM, BN, TM, TN, MINB>;
+  constexpr size_t smem = wide_smem<BM, BN>();
+  cudaError_t e = ensure_smem(reinterpret_cast<const void *>(fn), smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(fn, dim3((unsigned)tiles, 1, (unsigned)batch), dim3(kWideThreads), smem, s, M, N, K, A, B, C, sm);
+}
+
 template <int BK>
 cudaError_t launch_k(long long batch, long long M, long long N, long long K, const float2 *A, const float2 *B,
                      float2 *C, float2 *P, const OutMap &om, cudaStream_t s) {
@@ -379,6 +535,7 @@ cudaError_t launch_cgemm_fp32(long long batch, long long M, long long N, long lo
     const long long blocks = std::min<long long>((total + 255) / 256, (long long)num_sms() * 16);
     return launch_pdl(k_cgemm_small, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, m);
   }
+  if (P == nullptr && N > 32 && wide_ok(batch, M, N)) return launch_wide<128, 64, 8, 8, 2>(batch, M, N, K, A, B, C, m, s);
   if (K <= 8) return launch_k<8>(batch, M, N, K, A, B, C, P, m, s);
   return launch_k<16>(batch, M, N, K, A, B, C, P, m, s);
 }

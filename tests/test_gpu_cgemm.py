@@ -120,3 +120,25 @@ def test_block_diagonal_matricisation_is_the_batched_gemm():
     torch.cuda.synchronize()
     got = c.cpu().numpy().astype(np.complex128)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= TOL
+
+
+@pytest.mark.parametrize("shape", [(152, 128, 64, 16), (160, 65, 33, 1), (300, 129, 65, 17), (2, 1999, 1023, 19),
+                                   (64, 4096, 64, 8), (3, 1900, 1000, 33), (1, 2500, 1300, 50)])
+def test_cgemm_fp32_wide_tiles(shape):
+    """Shapes around the 128 x 64 tiles (whole ones, one row or column more, ragged ends of K, even and odd
+    rows for 16- and 8-byte copies), enough of them to take that form, against an FP64 product."""
+    err = _run(0, *shape)
+    assert err <= 1e-5
+
+
+@pytest.mark.parametrize("n,cols", [(12, 6), (13, 7)])
+def test_cgemm_fp32_wide_tiles_permuted_output(n, cols):
+    """The permuted epilogue of the 128 x 64 tiles through uniform blocks in plain FP32 (N = K = 2^cols)."""
+    from paper_2108_06831_gb300 import circuits as C
+    from oracle.statevector import simulate_state
+    tn = _tn()
+    c, _ = C.brickwork(n + 7, 3, 60 + n)
+    ctr = tn.Contractor(c, block_qubits=cols)
+    got = ctr.state().cpu().numpy()[0]
+    ref = simulate_state(c)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
