@@ -29,6 +29,7 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -419,7 +420,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgemm_tc(const __grid_constant_
 // epilogue (warp w owns TMEM lanes 32 (w mod 4)..+31).
 constexpr int kStreamThreads = 320;
 constexpr int kStreamMaxKTiles = 8;  // a single leading accumulator per tile stays accurate
-constexpr int kStgStride = 17;       // staging row stride (complex): rows fall in different banks
+
+// How an epilogue warp writes back a chunk of 32 rows x 16 complex columns of C (built on the host by
+// chunk_map).  The chunk's 9 local bits (4 column, 5 row) are enumerated by increasing stored position
+// as the bits of u; lane and iteration give u = 64 it + 2 lane (+ 1).  The chunk is staged at
+// row * 16 + (column ^ S(row)) with S linear over the row bits: s[k] is the staging contribution of u's
+// bit k (combined by XOR), g[k] its stored offset (combined by addition), and S is chosen so that both
+// the writes (lanes = rows) and the reads (lanes = bits 1-5 of u) of each half warp fall in distinct
+// banks.  Loads of index tables and bank conflicts of a padded staging were 1500 of the 4100 shared-
+// memory wavefronts of a tile, on a kernel bound by them.
+struct ChunkMap {
+  int row_swz[5];   // S of each row bit
+  int s[9];
+  long long g[9];
+  int pairs;        // u and u + 1 are adjacent in memory
+};
 
 // Split of one A stage from FP32 into three BF16 parts, in place: the FP32 tile is two 128-byte
 // boxes (K elements 32j..32j+31 of every row, 16-byte chunks swizzled by row mod 8); part p is a
@@ -471,7 +486,7 @@ template <int PREC>
 __global__ void __launch_bounds__(kStreamThreads, 1)
     k_cgemm_tc_stream(const __grid_constant__ TmaMaps maps, int k_tiles, int tiles_n, int tiles_m,
                       long long total_tiles, long long M, long long N2, float *__restrict__ C, int *status,
-                      const __grid_constant__ OutMap om) {
+                      const __grid_constant__ OutMap om, const __grid_constant__ ChunkMap cm) {
   using CF = Cfg<PREC>;
   pdl_wait();  // before any memory access or TMEM allocation: the previous kernel has completed
   pdl_trigger();
@@ -486,56 +501,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
   __shared__ int issued_parity[S];  // parity of the last TMA phase issued per stage, -1 if none
-  // Permuted epilogue: a warp stages 32 rows x 16 complex columns (one 32-float chunk of its
-  // rows) and writes them back in stored-index order.  The chunk's 9 local bits (5 row, 4
-  // column) are enumerated by increasing stored position (u); u -> staging offset and u ->
-  // stored offset are linear in u's bits, tabulated for u's low 5 and high 4 bits.
-  __shared__ float2 stage_c[4][32 * kStgStride];
-  __shared__ int sm_lo[32], sm_hi[16];
-  __shared__ long long g_lo[32], g_hi[16];
-  __shared__ int pairs_contig;
+  __shared__ float2 stage_c[4][32 * 16];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (!om.identity && threadIdx.x == 0) {
-    int lgn = 0;
-    while ((2ll << lgn) < N2) ++lgn;
-    // local bit b: b < 4 column bit b (stored at pos[b]); b >= 4 row bit b - 4 (pos[lgn + b - 4])
-    int spos[9], order[9];
-    for (int b = 0; b < 9; ++b) {
-      spos[b] = b < 4 ? om.pos[b] : om.pos[lgn + b - 4];
-      order[b] = b;
-    }
-    for (int i = 1; i < 9; ++i)  // insertion sort by stored position
-      for (int j = i; j > 0 && spos[order[j - 1]] > spos[order[j]]; --j) {
-        const int t = order[j];
-        order[j] = order[j - 1];
-        order[j - 1] = t;
-      }
-    auto contrib_s = [&](int b) { return b < 4 ? (1 << b) : (kStgStride << (b - 4)); };
-    for (int u = 0; u < 32; ++u) {
-      int so = 0;
-      long long go = 0;
-      for (int k = 0; k < 5; ++k)
-        if ((u >> k) & 1) {
-          so += contrib_s(order[k]);
-          go += 1ll << spos[order[k]];
-        }
-      sm_lo[u] = so;
-      g_lo[u] = go;
-    }
-    for (int u = 0; u < 16; ++u) {
-      int so = 0;
-      long long go = 0;
-      for (int k = 0; k < 4; ++k)
-        if ((u >> k) & 1) {
-          so += contrib_s(order[5 + k]);
-          go += 1ll << spos[order[5 + k]];
-        }
-      sm_hi[u] = so;
-      g_hi[u] = go;
-    }
-    pairs_contig = spos[order[0]] == 0 ? 1 : 0;
-  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
@@ -668,7 +636,17 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   } else {  // epilogue warps 6-9
     const int q = warp & 3;  // TMEM lane quarter this warp may access
     int lgn = 0;
-    while ((2ll << lgn) < N2) ++lgn;  // complex columns = 2^lgn
+    while ((2ll << lgn) < N2) ++lgn;  // complex columns = 2^lgn (with a permuted output)
+    float2 *stg = stage_c[q];
+    // this lane's part of the staging and stored offsets (u's bits 1-5)
+    int wr = 0, rd = 0;
+    long long go = 0;
+    for (int k = 0; k < 5; ++k)
+      if ((lane >> k) & 1) {
+        wr ^= (16 << k) ^ cm.row_swz[k];
+        rd ^= cm.s[k + 1];
+        go += cm.g[k + 1];
+      }
     long long li = 0;
     for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x, ++li) {
       const int ab = (int)(li & 1);
@@ -683,49 +661,30 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       decode(t, nt, mt, bz);
       const long long row0 = (long long)bz * M + (long long)mt * BM + q * 32;  // the warp's first row
       const uint32_t base = tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * 2 * BN);
-      float2 *stg = stage_c[q];
       for (int c = 0; c < BN; c += 32) {
         uint32_t r[32], e[32];
         tmem_ld32(base + BN + c, e);  // corrections
         tmem_ld32(base + c, r);       // leading product
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        float v[32];
 #pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(e[k]) + __uint_as_float(r[k]);
-        if (om.identity) {
-          // row-major: stage, then 8 lanes write each row's 128 bytes (4 rows per store)
-#pragma unroll
-          for (int k = 0; k < 16; ++k) stg[lane * kStgStride + k] = make_float2(v[2 * k], v[2 * k + 1]);
-          __syncwarp();
-          const float *cbase = C + ((long long)row0 * N2 + (long long)nt * BN + c);
-#pragma unroll
-          for (int it = 0; it < 8; ++it) {
-            const int pr = it * 32 + lane;  // pair index: row pr / 8, complex pair pr % 8
-            const int rr = pr >> 3, cc = 2 * (pr & 7);
-            const float2 x0 = stg[rr * kStgStride + cc], x1 = stg[rr * kStgStride + cc + 1];
-            *reinterpret_cast<float4 *>(const_cast<float *>(cbase) + (long long)rr * N2 + 2 * cc) =
-                make_float4(x0.x, x0.y, x1.x, x1.y);
-          }
-          __syncwarp();
-          continue;
-        }
-        // stored offset of everything but the chunk's local bits (lane row bits, 4 column bits)
-        const long long gbase = map_bits(om, (row0 << lgn) | ((long long)nt * (BN / 2) + c / 2), 0);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) stg[lane * kStgStride + k] = make_float2(v[2 * k], v[2 * k + 1]);
+        for (int k = 0; k < 16; ++k)
+          stg[wr ^ k] = make_float2(__uint_as_float(e[2 * k]) + __uint_as_float(r[2 * k]),
+                                    __uint_as_float(e[2 * k + 1]) + __uint_as_float(r[2 * k + 1]));
         __syncwarp();
-        float2 *C2 = reinterpret_cast<float2 *>(C);
+        // stored offset of everything but the chunk's local bits
+        float2 *C2 = reinterpret_cast<float2 *>(C) + go +
+                     (om.identity ? row0 * (N2 / 2) + nt * (BN / 2) + c / 2
+                                  : map_bits(om, (row0 << lgn) | ((long long)nt * (BN / 2) + c / 2), 0));
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
-          const int u = 64 * it + 2 * lane;  // even: u and u + 1 differ in the lowest sorted bit
-          const float2 x0 = stg[sm_lo[u & 31] + sm_hi[u >> 5]];
-          const float2 x1 = stg[sm_lo[(u + 1) & 31] + sm_hi[(u + 1) >> 5]];
-          const long long g0 = gbase + g_lo[u & 31] + g_hi[u >> 5];
-          if (pairs_contig) {
-            *reinterpret_cast<float4 *>(C2 + g0) = make_float4(x0.x, x0.y, x1.x, x1.y);
+          const int at = rd ^ ((it & 1) ? cm.s[6] : 0) ^ ((it & 2) ? cm.s[7] : 0) ^ ((it & 4) ? cm.s[8] : 0);
+          float2 *dst = C2 + ((it & 1) ? cm.g[6] : 0) + ((it & 2) ? cm.g[7] : 0) + ((it & 4) ? cm.g[8] : 0);
+          const float2 x0 = stg[at], x1 = stg[at ^ cm.s[0]];
+          if (cm.pairs) {
+            *reinterpret_cast<float4 *>(dst) = make_float4(x0.x, x0.y, x1.x, x1.y);
           } else {
-            C2[g0] = x0;
-            C2[gbase + g_lo[(u + 1) & 31] + g_hi[(u + 1) >> 5]] = x1;
+            dst[0] = x0;
+            dst[cm.g[0]] = x1;
           }
         }
         __syncwarp();
@@ -754,6 +713,46 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(kTmemCols));
   }
+}
+
+// The chunk's write-back for columns lgn (log2, with a permuted output) or N complex columns (row-major).
+void chunk_map(ChunkMap &cm, const OutMap &om, long long N) {
+  std::memset(&cm, 0, sizeof(cm));
+  int lgn = 0, order[9];
+  long long off[9];  // stored offset of local bit b: b < 4 column, else row
+  while ((1ll << lgn) < N) ++lgn;
+  for (int b = 0; b < 9; ++b) {
+    order[b] = b;
+    if (om.identity) off[b] = b < 4 ? 1ll << b : N << (b - 4);
+    else off[b] = 1ll << (b < 4 ? om.pos[b] : om.pos[lgn + b - 4]);
+  }
+  std::sort(order, order + 9, [&](int x, int y) { return off[x] < off[y]; });
+  // S: the row bits read by a half warp (bits 1-4 of u) take the column bits it does not read; the
+  // other row bits among the first four, the lanes of a write, take what is left of the column bits
+  bool col_read[4] = {false, false, false, false}, taken[4] = {false, false, false, false};
+  bool row_read[5] = {false, false, false, false, false};
+  for (int k = 1; k <= 4; ++k) (order[k] < 4 ? col_read[order[k]] : row_read[order[k] - 4]) = true;
+  int next = 0;
+  for (int r = 0; r < 5; ++r) {
+    if (!row_read[r]) continue;
+    while (col_read[next]) ++next;
+    cm.row_swz[r] = 1 << next;
+    if (r < 4) taken[next] = true;
+    ++next;
+  }
+  next = 0;
+  for (int r = 0; r < 4; ++r) {
+    if (row_read[r]) continue;
+    while (taken[next]) ++next;
+    cm.row_swz[r] = 1 << next;
+    taken[next] = true;
+  }
+  for (int k = 0; k < 9; ++k) {
+    const int b = order[k];
+    cm.s[k] = b < 4 ? 1 << b : (16 << (b - 4)) ^ cm.row_swz[b - 4];
+    cm.g[k] = off[b];
+  }
+  cm.pairs = off[order[0]] == 1;
 }
 
 // ------------------------------------------------------------------------------ prep kernels
@@ -915,9 +914,11 @@ cudaError_t run_tc(long long batch, long long M, long long N, long long K, const
       const int tiles_n = (int)((2 * N) / BN), tiles_m = (int)(M / BM);
       const long long total = (long long)tiles_n * tiles_m * batch;
       const long long grid = std::min<long long>(total, num_sms());
+      ChunkMap cm;
+      chunk_map(cm, om, N);
       return launch_pdl(k_cgemm_tc_stream<PREC>, dim3((unsigned)grid), dim3(kStreamThreads), smem, s, maps, k_tiles,
                         tiles_n, tiles_m, total, M, 2 * N, reinterpret_cast<float *>(C),
-                        static_cast<int *>(status_word_ptr()), om);
+                        static_cast<int *>(status_word_ptr()), om, cm);
     }
   }
   if constexpr (SPLIT_A && PREC == PREC_BF16) {
