@@ -133,18 +133,18 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   return d;
 }
 
-template <int PREC>
+template <int PREC, int N>
 __device__ __forceinline__ constexpr uint32_t instr_desc() {
   return (1u << 4)                                   // D: F32
          | ((uint32_t)Cfg<PREC>::kFmt << 7)          // A format
          | ((uint32_t)Cfg<PREC>::kFmt << 10)         // B format
-         | ((uint32_t)(BN >> 3) << 17)               // N
+         | ((uint32_t)(N >> 3) << 17)                // N
          | ((uint32_t)(BM >> 4) << 24);              // M
 }
 
-template <int PREC>
+template <int PREC, int N = BN>
 __device__ __forceinline__ void mma(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t acc) {
-  constexpr uint32_t idesc = instr_desc<PREC>();
+  constexpr uint32_t idesc = instr_desc<PREC, N>();
   if constexpr (PREC == PREC_TF32) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -580,16 +580,23 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t st = saddr(smem + (size_t)s * stage_bytes);
+          // products 0 and 1 share A's leading part, B's first two parts are adjacent in shared memory
+          // and the leading and correction accumulators in tensor memory: one MMA of 2 BN columns per
+          // K step does both, and reads A once.  The sums keep their order.
 #pragma unroll
-          for (int p = 0; p < CF::kProducts; ++p) {
+          for (int kk = 0; kk < KBYTES / (CF::kMmaK * CF::kElem); ++kk) {
+            const uint32_t off = kk * CF::kMmaK * CF::kElem;
+            mma<PREC, 2 * BN>(base, smem_desc(st + off), smem_desc(st + CF::kParts * kTileA + off),
+                              kt > 0 || kk > 0 ? 1u : 0u);
+          }
+#pragma unroll
+          for (int p = 2; p < CF::kProducts; ++p) {
             const uint32_t a_base = st + CF::pa(p) * kTileA;
             const uint32_t b_base = st + CF::kParts * kTileA + CF::pb(p) * kTileB;
 #pragma unroll
             for (int kk = 0; kk < KBYTES / (CF::kMmaK * CF::kElem); ++kk) {
               const uint32_t off = kk * CF::kMmaK * CF::kElem;
-              const uint32_t dst = p == 0 ? base : base + BN;
-              const bool acc = p == 0 ? (kt > 0 || kk > 0) : (kt > 0 || kk > 0 || p > 1);
-              mma<PREC>(dst, smem_desc(a_base + off), smem_desc(b_base + off), acc ? 1u : 0u);
+              mma<PREC>(base + BN, smem_desc(a_base + off), smem_desc(b_base + off), 1u);
             }
           }
           mma_issued = true;
