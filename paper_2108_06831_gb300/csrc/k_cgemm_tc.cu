@@ -416,9 +416,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgemm_tc(const __grid_constant_
 // stage ring runs on across tile boundaries, and the accumulators are double-buffered in
 // TMEM (leading + correction product per buffer, 2 x 2 x BN columns), so dedicated epilogue
 // warps drain tile i while tile i+1 is loaded, split and multiplied.
-// Warps 0-3: A split; warp 4: TMA; warp 5: TMEM allocation and MMA issue; warps 6-9:
+// The first split_warps: A split; then one for TMA, one for TMEM allocation and MMA issue, and four for the
 // epilogue (warp w owns TMEM lanes 32 (w mod 4)..+31).
-constexpr int kStreamThreads = 320;
+// Warps of the A split: four for TF32; eight for BF16, whose split reads, converts and writes three times
+// as much work per element (batch 64, 32768 x 64 x 64: 510 us with four, 444 with eight; TF32 399 and 403).
+template <int PREC>
+constexpr int split_warps() { return PREC == PREC_TF32 ? 4 : 8; }
+template <int PREC>
+constexpr int stream_threads() { return 32 * split_warps<PREC>() + 64 + 128; }  // + TMA, MMA and epilogue warps
 constexpr int kStreamMaxKTiles = 8;  // a single leading accumulator per tile stays accurate
 
 // How an epilogue warp writes back a chunk of 32 rows x 16 complex columns of C (built on the host by
@@ -438,14 +443,15 @@ struct ChunkMap {
 
 // Split of one A stage from FP32 into three BF16 parts, in place: the FP32 tile is two 128-byte
 // boxes (K elements 32j..32j+31 of every row, 16-byte chunks swizzled by row mod 8); part p is a
-// 128 x 64 BF16 tile at p x 16 KB (chunk d = K elements 8d..8d+7, same swizzle).  Each of the 128
-// converter threads first reads its 8 output chunks' sources, then (after a named barrier: the
+// 128 x 64 BF16 tile at p x 16 KB (chunk d = K elements 8d..8d+7, same swizzle).  Each of the
+// converter threads first reads its output chunks' sources, then (after a named barrier: the
 // parts overwrite the FP32 tile) writes x0 = bf16(x), x1 = bf16(x - x0), x2 = bf16(x - x0 - x1).
 __device__ __forceinline__ void split_bf16_in_place(unsigned char *st) {
-  float v[8][8];
+  constexpr int kSplitThreads = 32 * split_warps<PREC_BF16>(), kItems = 1024 / kSplitThreads;
+  float v[kItems][8];
 #pragma unroll
-  for (int it = 0; it < 8; ++it) {
-    const int item = threadIdx.x + kConvThreads * it, r = item >> 3, d = item & 7;
+  for (int it = 0; it < kItems; ++it) {
+    const int item = threadIdx.x + kSplitThreads * it, r = item >> 3, d = item & 7;
     const unsigned char *row = st + (d >> 2) * kTileA + r * 128;
     const int c0 = 2 * (d & 3);
     const float4 a = *reinterpret_cast<const float4 *>(row + ((c0 ^ (r & 7)) << 4));
@@ -453,10 +459,10 @@ __device__ __forceinline__ void split_bf16_in_place(unsigned char *st) {
     v[it][0] = a.x, v[it][1] = a.y, v[it][2] = a.z, v[it][3] = a.w;
     v[it][4] = b.x, v[it][5] = b.y, v[it][6] = b.z, v[it][7] = b.w;
   }
-  asm volatile("bar.sync 1, %0;" ::"n"(kConvThreads) : "memory");
+  asm volatile("bar.sync 1, %0;" ::"n"(kSplitThreads) : "memory");
 #pragma unroll
-  for (int it = 0; it < 8; ++it) {
-    const int item = threadIdx.x + kConvThreads * it, r = item >> 3, d = item & 7;
+  for (int it = 0; it < kItems; ++it) {
+    const int item = threadIdx.x + kSplitThreads * it, r = item >> 3, d = item & 7;
     uint32_t w[3][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -483,14 +489,14 @@ __device__ __forceinline__ void split_bf16_in_place(unsigned char *st) {
 }
 
 template <int PREC>
-__global__ void __launch_bounds__(kStreamThreads, 1)
+__global__ void __launch_bounds__(stream_threads<PREC>(), 1)
     k_cgemm_tc_stream(const __grid_constant__ TmaMaps maps, int k_tiles, int tiles_n, int tiles_m,
                       long long total_tiles, long long M, long long N2, float *__restrict__ C, int *status,
                       const __grid_constant__ OutMap om, const __grid_constant__ ChunkMap cm) {
   using CF = Cfg<PREC>;
   pdl_wait();  // before any memory access or TMEM allocation: the previous kernel has completed
   pdl_trigger();
-  constexpr int S = CF::kStages;
+  constexpr int S = CF::kStages, kSplitWarps = split_warps<PREC>(), kSplitThreads = 32 * kSplitWarps;
   constexpr int stage_bytes = CF::kParts * (kTileA + kTileB);
   // A arrives as FP32: one 128-byte box per row and K tile for TF32, two for BF16 (64 elements)
   constexpr int a_boxes = PREC == PREC_TF32 ? 1 : 2;
@@ -507,7 +513,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&conv[s], kConvThreads);
+      mbar_init(&conv[s], kSplitThreads);
       mbar_init(&empty[s], 1);
       issued_parity[s] = -1;
     }
@@ -519,7 +525,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 5) {
+  if (warp == kSplitWarps + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_base)),
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -528,7 +534,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_d = tmem_base;
-  bool mma_issued = false;  // warp 5 lane 0: at least one MMA was issued
+  bool mma_issued = false;  // MMA warp lane 0: at least one MMA was issued
 
   auto aborted = [&]() { return *reinterpret_cast<volatile int *>(&abort_flag) != 0; };
   auto decode = [&](long long t, int &nt, int &mt, int &bz) {
@@ -538,7 +544,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     bz = (int)(r / tiles_m);
   };
 
-  if (warp == 4) {
+  if (warp == kSplitWarps) {
     if (lane == 0) {  // TMA producer
       long long g = 0;
       for (long long t = blockIdx.x; t < total_tiles && !aborted(); t += gridDim.x) {
@@ -560,7 +566,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         }
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == kSplitWarps + 1) {
     if (lane == 0) {  // MMA issuer
       long long g = 0, li = 0;
       for (long long t = blockIdx.x; t < total_tiles && !aborted(); t += gridDim.x, ++li) {
@@ -609,7 +615,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         mma_commit(&acc_full[ab]);
       }
     }
-  } else if (warp < 4) {  // A split, as in k_cgemm_tc
+  } else if (warp < kSplitWarps) {  // A split, as in k_cgemm_tc
     long long g = 0;
     for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
       bool ok = true;
@@ -623,7 +629,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
           float4 *hi = reinterpret_cast<float4 *>(smem + (size_t)s * stage_bytes);
           float4 *lo = reinterpret_cast<float4 *>(smem + (size_t)s * stage_bytes + kTileA);
 #pragma unroll 4
-          for (int c = threadIdx.x; c < kTileA / 16; c += kConvThreads) {
+          for (int c = threadIdx.x; c < kTileA / 16; c += kSplitThreads) {
             const float4 v = hi[c];
             const float4 h = make_float4(tf32_rna(v.x), tf32_rna(v.y), tf32_rna(v.z), tf32_rna(v.w));
             lo[c] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
@@ -640,7 +646,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         break;
       }
     }
-  } else {  // epilogue warps 6-9
+  } else {  // epilogue warps
     const int q = warp & 3;  // TMEM lane quarter this warp may access
     int lgn = 0;
     while ((2ll << lgn) < N2) ++lgn;  // complex columns = 2^lgn (with a permuted output)
@@ -709,14 +715,14 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     if (threadIdx.x == 0)
       for (int s = 0; s < S; ++s)
         if (issued_parity[s] >= 0) mbar_wait(&full[s], (uint32_t)issued_parity[s], nullptr);
-    if (warp == 5 && lane == 0 && mma_issued) {
+    if (warp == kSplitWarps + 1 && lane == 0 && mma_issued) {
       mma_commit(&drain);
       mbar_wait(&drain, 0, nullptr);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
   }
-  if (warp == 5) {
+  if (warp == kSplitWarps + 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(kTmemCols));
   }
@@ -923,7 +929,7 @@ cudaError_t run_tc(long long batch, long long M, long long N, long long K, const
       const long long grid = std::min<long long>(total, num_sms());
       ChunkMap cm;
       chunk_map(cm, om, N);
-      return launch_pdl(k_cgemm_tc_stream<PREC>, dim3((unsigned)grid), dim3(kStreamThreads), smem, s, maps, k_tiles,
+      return launch_pdl(k_cgemm_tc_stream<PREC>, dim3((unsigned)grid), dim3(stream_threads<PREC>()), smem, s, maps, k_tiles,
                         tiles_n, tiles_m, total, M, 2 * N, reinterpret_cast<float *>(C),
                         static_cast<int *>(status_word_ptr()), om, cm);
     }
