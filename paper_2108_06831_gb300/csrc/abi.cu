@@ -152,6 +152,135 @@ tn_status call_mats(const tn_plan *p, const double *params, void *ws, cudaStream
   return TN_OK;
 }
 
+double lean_weight(const TnGate &g) {
+  switch (g.kind) {
+    case TN_GATE_MAT2: return 4.0;
+    case TN_GATE_U3: case TN_GATE_RX: case TN_GATE_RY: case TN_GATE_H: case TN_GATE_Y: case TN_GATE_SX: case TN_GATE_SY:
+    case TN_GATE_SW: case TN_GATE_MAT1:
+      return 1.0;
+    default: return 0.0;
+  }
+}
+
+// Passes, tables and generated kernels of a state plan whose sizes (n, batch, T, K, ..) are set.  On
+// failure everything but p itself has been freed.
+tn_status build_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, std::string &err) {
+  // Precontracted blocks cost a per-call FP64 product when the circuit reads parameters; below
+  // kFuseMinQubitsParam qubits that costs more than the smaller state saves in the passes.
+  const bool fuse = !(o.flags & TN_PLAN_NO_FUSION) && (c->n_params == 0 || c->n >= kFuseMinQubitsParam);
+  const tn_circuit fwd_circ = push_phases(fuse ? fuse_pairs(*c, p->fused) : *c, p->fused);
+  for (const TnGate &g : fwd_circ.gates) p->n_fused += g.kind == KIND_F2 ? 1 : 0;
+  tn_status st = build_pass_plan(fwd_circ, p->T, p->K, false, p->slots, p->fwd, err);
+  // the adjoint sweep stages two tiles (psi, lambda), double-buffered: at most 2^11 amplitudes each
+  const int T_bwd = std::min(p->T, 11);
+  if (st == TN_OK && o.target == TN_TARGET_EXPECTATION)
+    st = build_pass_plan(*c, T_bwd, std::min(T_bwd, 4), true, p->slots, p->bwd, err);
+  if (st != TN_OK) {
+    set_error("planner: %s", err.c_str());
+    return st;
+  }
+  p->mstride = 0;
+  if (!p->slots.empty()) {
+    const MatSlot &l = p->slots.back();
+    p->mstride = l.offset + shape_units(l.shape);
+  }
+  p->mstride = (p->mstride + 1) & ~1;
+  p->param_dependent = c->n_params > 0;
+
+  // workspace layout
+  size_t off = 0;
+  const size_t state_bytes = ((size_t)sizeof(float2) << c->n) * (size_t)o.batch;
+  if (p->param_dependent) {
+    p->ws_mats = off;
+    off = align_up(off + (size_t)p->mstride * sizeof(float2) * (size_t)o.batch);
+  }
+  if (o.target != TN_TARGET_STATE) {
+    p->ws_psi = off;
+    off = align_up(off + state_bytes);
+  }
+  if (o.target == TN_TARGET_EXPECTATION) {
+    p->ws_lam = off;
+    off = align_up(off + state_bytes);
+    p->ws_part = off;
+    off = align_up(off + (size_t)o.batch * kMaxRedPasses * 512 * sizeof(double));
+  }
+  p->ws_bytes = off;
+
+  if (p->host_only && getenv("TNQ_JIT_COMPILE_CHECK") && !(o.flags & TN_PLAN_NO_SPECIALIZE) && jit_supported(*p)) {
+    // generate and compile the specialised kernels without loading them (no GPU needed)
+    std::vector<int> kinds(p->fwd.ops.size());
+    for (size_t i = 0; i < kinds.size(); ++i) kinds[i] = fwd_circ.gates[(size_t)p->fwd.op_gate[i]].kind;
+    std::string jerr;
+    tn_status u = jit_build(*p, kinds, false, true, jerr);
+    if (u == TN_OK && jit_bwd_supported(*p)) {
+      std::vector<int> bk(p->bwd.ops.size());
+      for (size_t i = 0; i < bk.size(); ++i) bk[i] = c->gates[(size_t)p->bwd.op_gate[i]].kind;
+      u = jit_build(*p, bk, true, true, jerr);
+    }
+    if (u != TN_OK) {
+      set_error("plan-specialised kernels: %s", jerr.c_str());
+      return u;
+    }
+  }
+  if (!p->host_only) {
+    tn_status u = TN_OK;
+    cudaError_t de = cudaGetDevice(&p->device);
+    if (de != cudaSuccess) u = cuda_fail(de, "cudaGetDevice");
+    if (u == TN_OK) {  // device copy in the order the materialisation kernel reads (fused blocks first)
+      std::vector<MatSlot> ordered = p->slots;
+      p->n_fused_slots = order_slots_fused_first(ordered);
+      u = upload(ordered, &p->d_slots);
+    }
+    if (u == TN_OK && !p->fused.empty()) u = upload(p->fused, &p->d_fused);
+    if (u == TN_OK) u = upload(p->fwd.passes, &p->d_fwd_pass);
+    if (u == TN_OK) u = upload(p->fwd.phases, &p->d_fwd_phase);
+    if (u == TN_OK) u = upload(p->fwd.ops, &p->d_fwd_ops);
+    if (u == TN_OK) u = upload(p->bwd.passes, &p->d_bwd_pass);
+    if (u == TN_OK) u = upload(p->bwd.phases, &p->d_bwd_phase);
+    if (u == TN_OK) u = upload(p->bwd.ops, &p->d_bwd_ops);
+    if (u == TN_OK) u = upload(p->bwd.grads, &p->d_bwd_grads);
+    if (u == TN_OK && !p->param_dependent && p->mstride > 0) {
+      cudaError_t e = cudaMalloc((void **)&p->d_fixed_mats, (size_t)p->mstride * sizeof(float2));
+      if (e != cudaSuccess) {
+        set_error("cudaMalloc of the fixed gate table: %s", cudaGetErrorString(e));
+        u = TN_ERR_OOM;
+      } else {
+        e = launch_materialize(p->d_slots, (int)p->slots.size(), p->n_fused_slots, p->d_fused, nullptr, 0, 1, p->mstride,
+                               reinterpret_cast<float2 *>(p->d_fixed_mats), 0);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) u = cuda_fail(e, "fixed gate table");
+      }
+    }
+    if (u == TN_OK && !(o.flags & TN_PLAN_NO_SPECIALIZE) && jit_supported(*p)) {
+      std::vector<int> kinds(p->fwd.ops.size());
+      for (size_t i = 0; i < kinds.size(); ++i) kinds[i] = fwd_circ.gates[(size_t)p->fwd.op_gate[i]].kind;
+      std::string jerr;
+      u = jit_build(*p, kinds, false, false, jerr);
+      if (u == TN_OK && !p->param_dependent && p->d_fixed_mats) {
+        // fixed angles: each pass's constant table is filled once
+        for (size_t i = 0; i < p->jit_cm_ptr.size() && u == TN_OK; ++i)
+          if (p->jit_cm_ptr[i] && p->jit_cm_bytes[i]) {
+            cudaError_t e = cudaMemcpy(p->jit_cm_ptr[i], p->d_fixed_mats + 2 * (size_t)p->fwd.passes[i].mat_begin,
+                                       p->jit_cm_bytes[i], cudaMemcpyDeviceToDevice);
+            if (e != cudaSuccess) u = cuda_fail(e, "generated kernels' matrix tables");
+          }
+      }
+      if (u == TN_OK && jit_bwd_supported(*p)) {
+        std::vector<int> bk(p->bwd.ops.size());
+        for (size_t i = 0; i < bk.size(); ++i) bk[i] = c->gates[(size_t)p->bwd.op_gate[i]].kind;
+        u = jit_build(*p, bk, true, false, jerr);
+      }
+      if (u != TN_OK) set_error("plan-specialised kernels: %s", jerr.c_str());
+    }
+    if (u != TN_OK) {
+      jit_release(*p);
+      free_plan_device(p);
+      return u;
+    }
+  }
+  return TN_OK;
+}
+
 tn_status common_checks(const tn_plan *p) {
   TN_CHECK_ARG(p != nullptr, "plan is NULL");
   TN_CHECK_ARG(!p->host_only, "plan was built with TN_PLAN_HOST_ONLY and cannot run");
@@ -353,120 +482,43 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
     *out = p;
     return TN_OK;
   }
-  // Precontracted blocks cost a per-call FP64 product when the circuit reads parameters; below
-  // kFuseMinQubitsParam qubits that costs more than the smaller state saves in the passes.
-  const bool fuse = !(o.flags & TN_PLAN_NO_FUSION) && (c->n_params == 0 || c->n >= kFuseMinQubitsParam);
-  const tn_circuit fwd_circ = push_phases(fuse ? fuse_pairs(*c, p->fused) : *c, p->fused);
-  for (const TnGate &g : fwd_circ.gates) p->n_fused += g.kind == KIND_F2 ? 1 : 0;
-  tn_status st = build_pass_plan(fwd_circ, T, K, false, p->slots, p->fwd, err);
-  // the adjoint sweep stages two tiles (psi, lambda), double-buffered: at most 2^11 amplitudes each
-  const int T_bwd = std::min(T, 11);
-  if (st == TN_OK && o.target == TN_TARGET_EXPECTATION)
-    st = build_pass_plan(*c, T_bwd, std::min(T_bwd, 4), true, p->slots, p->bwd, err);
-  if (st != TN_OK) {
-    set_error("planner: %s", err.c_str());
-    delete p;
-    return st;
-  }
-  p->mstride = 0;
-  if (!p->slots.empty()) {
-    const MatSlot &l = p->slots.back();
-    p->mstride = l.offset + shape_units(l.shape);
-  }
-  p->mstride = (p->mstride + 1) & ~1;
-  p->param_dependent = c->n_params > 0;
-
-  // workspace layout
-  size_t off = 0;
-  const size_t state_bytes = ((size_t)sizeof(float2) << c->n) * (size_t)o.batch;
-  if (p->param_dependent) {
-    p->ws_mats = off;
-    off = align_up(off + (size_t)p->mstride * sizeof(float2) * (size_t)o.batch);
-  }
-  if (o.target != TN_TARGET_STATE) {
-    p->ws_psi = off;
-    off = align_up(off + state_bytes);
-  }
-  if (o.target == TN_TARGET_EXPECTATION) {
-    p->ws_lam = off;
-    off = align_up(off + state_bytes);
-    p->ws_part = off;
-    off = align_up(off + (size_t)o.batch * kMaxRedPasses * 512 * sizeof(double));
-  }
-  p->ws_bytes = off;
-
-  if (p->host_only && getenv("TNQ_JIT_COMPILE_CHECK") && !(o.flags & TN_PLAN_NO_SPECIALIZE) && jit_supported(*p)) {
-    // generate and compile the specialised kernels without loading them (no GPU needed)
-    std::vector<int> kinds(p->fwd.ops.size());
-    for (size_t i = 0; i < kinds.size(); ++i) kinds[i] = fwd_circ.gates[(size_t)p->fwd.op_gate[i]].kind;
-    std::string jerr;
-    tn_status u = jit_build(*p, kinds, false, true, jerr);
-    if (u == TN_OK && jit_bwd_supported(*p)) {
-      std::vector<int> bk(p->bwd.ops.size());
-      for (size_t i = 0; i < bk.size(); ++i) bk[i] = c->gates[(size_t)p->bwd.op_gate[i]].kind;
-      u = jit_build(*p, bk, true, true, jerr);
-    }
-    if (u != TN_OK) {
-      set_error("plan-specialised kernels: %s", jerr.c_str());
-      delete p;
-      return u;
-    }
-  }
-  if (!p->host_only) {
-    TN_CUDA(cudaGetDevice(&p->device), "cudaGetDevice");
-    tn_status u = TN_OK;
-    if (u == TN_OK) {  // device copy in the order the materialisation kernel reads (fused blocks first)
-      std::vector<MatSlot> ordered = p->slots;
-      p->n_fused_slots = order_slots_fused_first(ordered);
-      u = upload(ordered, &p->d_slots);
-    }
-    if (u == TN_OK && !p->fused.empty()) u = upload(p->fused, &p->d_fused);
-    if (u == TN_OK) u = upload(p->fwd.passes, &p->d_fwd_pass);
-    if (u == TN_OK) u = upload(p->fwd.phases, &p->d_fwd_phase);
-    if (u == TN_OK) u = upload(p->fwd.ops, &p->d_fwd_ops);
-    if (u == TN_OK) u = upload(p->bwd.passes, &p->d_bwd_pass);
-    if (u == TN_OK) u = upload(p->bwd.phases, &p->d_bwd_phase);
-    if (u == TN_OK) u = upload(p->bwd.ops, &p->d_bwd_ops);
-    if (u == TN_OK) u = upload(p->bwd.grads, &p->d_bwd_grads);
-    if (u == TN_OK && !p->param_dependent && p->mstride > 0) {
-      cudaError_t e = cudaMalloc((void **)&p->d_fixed_mats, (size_t)p->mstride * sizeof(float2));
-      if (e != cudaSuccess) {
-        set_error("cudaMalloc of the fixed gate table: %s", cudaGetErrorString(e));
-        u = TN_ERR_OOM;
-      } else {
-        e = launch_materialize(p->d_slots, (int)p->slots.size(), p->n_fused_slots, p->d_fused, nullptr, 0, 1, p->mstride,
-                               reinterpret_cast<float2 *>(p->d_fixed_mats), 0);
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) u = cuda_fail(e, "fixed gate table");
-      }
-    }
-    if (u == TN_OK && !(o.flags & TN_PLAN_NO_SPECIALIZE) && jit_supported(*p)) {
-      std::vector<int> kinds(p->fwd.ops.size());
-      for (size_t i = 0; i < kinds.size(); ++i) kinds[i] = fwd_circ.gates[(size_t)p->fwd.op_gate[i]].kind;
-      std::string jerr;
-      u = jit_build(*p, kinds, false, false, jerr);
-      if (u == TN_OK && !p->param_dependent && p->d_fixed_mats) {
-        // fixed angles: each pass's constant table is filled once
-        for (size_t i = 0; i < p->jit_cm_ptr.size() && u == TN_OK; ++i)
-          if (p->jit_cm_ptr[i] && p->jit_cm_bytes[i]) {
-            cudaError_t e = cudaMemcpy(p->jit_cm_ptr[i], p->d_fixed_mats + 2 * (size_t)p->fwd.passes[i].mat_begin,
-                                       p->jit_cm_bytes[i], cudaMemcpyDeviceToDevice);
-            if (e != cudaSuccess) u = cuda_fail(e, "generated kernels' matrix tables");
-          }
-      }
-      if (u == TN_OK && jit_bwd_supported(*p)) {
-        std::vector<int> bk(p->bwd.ops.size());
-        for (size_t i = 0; i < bk.size(); ++i) bk[i] = c->gates[(size_t)p->bwd.op_gate[i]].kind;
-        u = jit_build(*p, bk, true, false, jerr);
-      }
-      if (u != TN_OK) set_error("plan-specialised kernels: %s", jerr.c_str());
-    }
-    if (u != TN_OK) {
+  // A plan of few warps (see kLeanWarps) runs its forward passes from a second, lean plan; the first
+  // then only serves the batched executor's tables and needs no generated kernels.
+  double mixing = 0.0;  // gates that mix amplitudes: permutations and diagonal gates are cheap either way
+  for (const TnGate &g : c->gates) mixing += lean_weight(g);
+  const bool lean = o.target != TN_TARGET_EXPECTATION && !p->host_only && !(o.flags & TN_PLAN_NO_SPECIALIZE) &&
+                    T >= kLowBits + 2 && c->n < kBatchDirectMinQubits && mixing >= kLeanGates &&
+                    (c->n_params == 0 || c->n < kFuseMinQubitsParam) &&
+                    std::ldexp((double)o.batch, c->n - 9) < kLeanWarps * (double)num_sms();
+  tn_plan_opts o_main = o;
+  if (lean) o_main.flags |= TN_PLAN_NO_SPECIALIZE;
+  tn_status st = build_passes(c, o_main, p, err);
+  if (st == TN_OK && lean) {
+    tn_plan *q = new tn_plan();
+    q->n = p->n;
+    q->batch = p->batch;
+    q->n_params = p->n_params;
+    q->n_gates = p->n_gates;
+    q->init = p->init;
+    q->opts = o;
+    q->host_only = false;
+    q->device = -1;
+    q->T = T;
+    q->K = c->n <= 12 && T <= 12 ? kLeanReg : kLeanReg + 1;  // at most 1024 threads
+    q->is_lean = true;
+    st = build_passes(c, o, q, err);
+    if (st == TN_OK) {
+      p->lean = q;
+      p->ws_bytes = std::max(p->ws_bytes, q->ws_bytes);
+    } else {
+      delete q;
       jit_release(*p);
       free_plan_device(p);
-      delete p;
-      return u;
     }
+  }
+  if (st != TN_OK) {
+    delete p;
+    return st;
   }
   *out = p;
   return TN_OK;
@@ -520,6 +572,10 @@ tn_status tn_plan_get_stats(const tn_plan *p, tn_plan_stats *st) {
     st->q428_launches = q428_launches(p->q428);
     return TN_OK;
   }
+  if (p->lean) p = p->lean;  // the plan that tn_contract_state runs
+  st->n_passes = (int)p->fwd.passes.size();
+  st->n_phases = (int)p->fwd.phases.size();
+  st->n_ops = (long long)p->fwd.ops.size();
   st->tile_qubits = p->T;
   st->reg_qubits = p->K;
   st->flops = p->fwd.flops;
@@ -574,6 +630,7 @@ void tn_free_plan(tn_plan *p) {
     delete p;
     return;
   }
+  if (p->lean) tn_free_plan(p->lean);
   jit_release(*p);
   if (!p->host_only) free_plan_device(p);
   delete p;
@@ -725,6 +782,7 @@ tn_status tn_contract_state(const tn_plan *p, const double *params_dev, void *st
             "block contraction");
     return TN_OK;
   }
+  if (p->lean) p = p->lean;
   const float2 *mats = nullptr;
   long long mstride = 0;
   st = call_mats(p, params_dev, workspace_dev, cs, &mats, &mstride);
@@ -741,6 +799,7 @@ tn_status tn_contract_amplitudes(const tn_plan *p, const double *params_dev, con
   TN_CHECK_ARG(n_bitstrings >= 0, "n_bitstrings < 0");
   TN_CHECK_ARG(n_bitstrings == 0 || (bitstrings_dev != nullptr && amps_dev != nullptr), "NULL device pointer");
   TN_CHECK_ARG(workspace_dev != nullptr, "workspace_dev is NULL");
+  if (p->lean) p = p->lean;
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(s);
   const float2 *mats = nullptr;
   long long mstride = 0;

@@ -325,7 +325,9 @@ void emit_op(Emitter &E, const OpDesc &op, int kind) {
 bool jit_const_mats(const tn_plan &p) {
   if (const char *e = getenv("TNQ_JIT_CONST"))
     if (atoi(e) == 0) return false;
-  return !p.param_dependent || p.batch == 1;
+  // per-call tables of smaller states are staged in shared memory: the copies into the constant tables, one
+  // before each pass, cost more than they save (16 qubits depth 10: 47 us with them, 37 without; 22: 159, 170)
+  return !p.param_dependent || (p.batch == 1 && p.n >= kConstMinQubits);
 }
 
 namespace {
@@ -352,6 +354,7 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
   // the SMs across streams); two when each batch element's entries are staged in shared memory (the
   // 64-set adjoint configuration's forward passes ran 8% slower at three)
   int min_blocks = cmem ? 3 : 2;
+  if (p.is_lean) min_blocks = std::max(1, std::min(4, 1024 / NTHR));
   if (const char *mb = getenv("TNQ_JIT_MIN_BLOCKS")) min_blocks = std::max(1, std::min(4, atoi(mb)));
   if (cmem) {
     snprintf(buf, sizeof buf, "__constant__ float4 tnq_cm%d[%d];", pi, std::max(1, mat_n / 2));
@@ -975,7 +978,7 @@ tn_status compile_cubin(const std::string &src, std::string &cubin, std::string 
 bool jit_supported(const tn_plan &p) {
   if (p.fwd.passes.empty()) return false;
   for (const PassDesc &pd : p.fwd.passes)
-    if (pd.K != 4 || pd.T < kLowBits + 2) return false;
+    if ((pd.K != 4 && !p.is_lean) || pd.K < 2 || pd.T < kLowBits + 2) return false;
   return true;
 }
 

@@ -10,13 +10,19 @@ namespace tnq {
 
 // Gate tensors are built once per call from the parameters (angles in FP64, entries stored as
 // complex64).  The slot array lists the fused blocks (KIND_F2) first.  Few fused blocks (small
-// batches): each block and batch element takes one warp -- lane m evaluates member m's matrix
-// embedded as a 4x4, then lanes 0..15 form the product one entry each, member by member.  Many
-// (kFusedPerThread or more): one thread each, members applied in turn to a 4x4 held by the thread
-// (all lanes busy; FP64 throughput is what bounds this on GB300).  Either way the product is
-// stored in the packed layout (SHAPE_M4X).  Every other slot and batch element takes one thread.
-constexpr int kMatWarps = 4;
+// batches): each block and batch element takes one warp -- lanes evaluate the members' sines and
+// cosines one angle each, lane m embeds member m's matrix as a 4x4, then lanes 0..15 form the product
+// one entry each, member by member.  Many (kFusedPerThread or more): one thread each, members applied
+// in turn to a 4x4 held by the thread (all lanes busy).  Either way the product is stored in the packed
+// layout (SHAPE_M4X).  Every other slot and batch element takes one thread, or four (one per angle)
+// where there are few.
+// Bound: FP64, two operations per SM and clock, so a warp's instruction takes 16 clocks of its SM and a
+// sincos about a microsecond with nothing beside it.  Hence one warp per CTA: the warps spread over the
+// SMs instead of queueing on one FP64 unit.  Whole calls with four warps per CTA and one thread per
+// slot or member, and now: 10-qubit brickwork of depth 8, 16 sets 14.4 and 12.4 us; 16 qubits, depth 10,
+// one set 37 and 33 us; 22 qubits 159 and 155 us.
 constexpr long long kFusedPerThread = 1024;  // fused blocks x batch from which each takes one thread
+constexpr long long kSpreadSlots = 4096;     // other slots x batch up to which each takes four threads
 
 // One regular slot (one gate's matrix) for one batch element; prow: its parameters (may be NULL).
 __device__ void materialize_one(const MatSlot &s, const double *prow, float2 *table) {
@@ -24,23 +30,51 @@ __device__ void materialize_one(const MatSlot &s, const double *prow, float2 *ta
   for (int a = 0; a < 3; ++a)
     for (int q = 0; q < 2; ++q)
       if (s.pidx[a][q] >= 0) ang[a] += prow[s.pidx[a][q]];
-  double tmp[32];
+  double tmp[32], x[3] = {0.0, 0.0, 0.0}, sn[3], cs[3];
   float ent[32];
-  const int n = slot_entries(s, ang, tmp, ent);
+  const int nx = gate_trig(s.kind, ang, x);
+  for (int a = 0; a < nx; ++a) sincos2(x[a], &sn[a], &cs[a]);
+  const int n = slot_entries(s, sn, cs, tmp, ent);
   float2 *dst = table + s.offset;
   for (int i = 0; i < n; ++i) dst[i] = make_float2(ent[2 * i], ent[2 * i + 1]);
 }
 
-__global__ void __launch_bounds__(32 * kMatWarps) k_materialize(const MatSlot *__restrict__ slots, int n_slots,
+// One regular slot by four consecutive lanes: lane a evaluates angle a's sine and cosine, lane 0 composes.
+__device__ void materialize_spread(const MatSlot &s, const double *prow, float2 *table, int lane, bool live) {
+  double x[3] = {0.0, 0.0, 0.0}, sn = 0.0, cs = 0.0;
+  const int a = lane & 3;
+  if (live) {
+    double ang[3] = {s.angle[0], s.angle[1], s.angle[2]};
+    for (int k = 0; k < 3; ++k)
+      for (int q = 0; q < 2; ++q)
+        if (s.pidx[k][q] >= 0) ang[k] += prow[s.pidx[k][q]];
+    if (a < gate_trig(s.kind, ang, x)) sincos2(a == 0 ? x[0] : a == 1 ? x[1] : x[2], &sn, &cs);
+  }
+  double sv[3], cv[3];
+  for (int k = 0; k < 3; ++k) {
+    sv[k] = __shfl_sync(0xFFFFFFFFu, sn, (lane & ~3) + k);
+    cv[k] = __shfl_sync(0xFFFFFFFFu, cs, (lane & ~3) + k);
+  }
+  if (!live || a != 0) return;
+  double tmp[32];
+  float ent[32];
+  const int n = slot_entries(s, sv, cv, tmp, ent);
+  float2 *dst = table + s.offset;
+  for (int i = 0; i < n; ++i) dst[i] = make_float2(ent[2 * i], ent[2 * i + 1]);
+}
+
+__global__ void __launch_bounds__(32) k_materialize(const MatSlot *__restrict__ slots, int n_slots,
                                                                int n_fused_slots,
                                                                const FusedMember *__restrict__ fused,
                                                                const double *__restrict__ params, int n_params,
                                                                int batch, long long mstride, float2 *__restrict__ out,
-                                                               int fused_per_thread) {
-  __shared__ double emb[kMatWarps][kMaxFusedMembers][32];
-  __shared__ double acc[kMatWarps][2][32];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long gw = (long long)blockIdx.x * kMatWarps + w;  // global warp
+                                                               int fused_per_thread, int spread) {
+  __shared__ double emb[kMaxFusedMembers][32];
+  __shared__ double acc[2][32];
+  __shared__ double trig[kMaxFusedMembers][3][2];  // sine, cosine
+  __shared__ int shape[kMaxFusedMembers];  // which entries of a row of emb can be nonzero: 0 all, 1 diagonal, 2 on a, 3 on b
+  const int lane = threadIdx.x;
+  const long long gw = blockIdx.x;
   if (fused_per_thread) {
     // many fused blocks (large batches): one thread each, every lane busy in FP64
     const long long n_ft = (long long)n_fused_slots * batch;
@@ -77,28 +111,46 @@ __global__ void __launch_bounds__(32 * kMatWarps) k_materialize(const MatSlot *_
     float2 *dst = out + (long long)b * mstride + s.offset;
     const double *prow = params ? params + (long long)b * n_params : nullptr;
     const int cnt = s.fuse_count;
-    if (lane < cnt) fused_embed(fused[s.fuse_begin + lane], prow, emb[w][lane]);
-    acc[w][0][lane] = (lane & 1) == 0 && ((lane >> 1) % 5) == 0 ? 1.0 : 0.0;  // identity
+    for (int it = lane; it < 3 * cnt; it += 32) {
+      const int m = it / 3, a = it - 3 * m;
+      const FusedMember &f = fused[s.fuse_begin + m];
+      double ang[3] = {f.angle[0], f.angle[1], f.angle[2]}, x[3] = {0.0, 0.0, 0.0};
+      for (int k = 0; k < 3; ++k)
+        for (int q = 0; q < 2; ++q)
+          if (f.pidx[k][q] >= 0 && prow) ang[k] += prow[f.pidx[k][q]];
+      if (a < gate_trig(f.kind, ang, x)) sincos2(a == 0 ? x[0] : a == 1 ? x[1] : x[2], &trig[m][a][0], &trig[m][a][1]);
+    }
+    acc[0][lane] = (lane & 1) == 0 && ((lane >> 1) % 5) == 0 ? 1.0 : 0.0;  // identity
+    __syncwarp();
+    if (lane < cnt) {
+      double sn[3], cs[3];
+      for (int a = 0; a < 3; ++a) sn[a] = trig[lane][a][0], cs[a] = trig[lane][a][1];
+      const FusedMember &f = fused[s.fuse_begin + lane];
+      fused_embed(f, sn, cs, emb[lane]);
+      shape[lane] = gate_nqubits(f.kind) == 1 ? (f.role == ROLE_A ? 2 : 3) : f.kind == TN_GATE_CZ || f.kind == TN_GATE_CP ? 1 : 0;
+    }
     __syncwarp();
     int cur = 0;
     for (int m = 0; m < cnt; ++m) {  // acc <- emb[m] * acc
       if (lane < 16) {
         const int i = lane >> 2, j = lane & 3;
         double re = 0.0, im = 0.0;
-        for (int q = 0; q < 4; ++q) {
-          const double xr = emb[w][m][2 * (4 * i + q)], xi = emb[w][m][2 * (4 * i + q) + 1];
-          const double yr = acc[w][cur][2 * (4 * q + j)], yi = acc[w][cur][2 * (4 * q + j) + 1];
+        const int sh = shape[m], terms = sh == 0 ? 4 : sh == 1 ? 1 : 2;
+        for (int k = 0; k < terms; ++k) {  // the others are zero
+          const int q = sh == 0 ? k : sh == 1 ? i : sh == 2 ? 2 * k + (i & 1) : (i & 2) + k;
+          const double xr = emb[m][2 * (4 * i + q)], xi = emb[m][2 * (4 * i + q) + 1];
+          const double yr = acc[cur][2 * (4 * q + j)], yi = acc[cur][2 * (4 * q + j) + 1];
           re += xr * yr - xi * yi;
           im += xr * yi + xi * yr;
         }
-        acc[w][cur ^ 1][2 * lane] = re;
-        acc[w][cur ^ 1][2 * lane + 1] = im;
+        acc[cur ^ 1][2 * lane] = re;
+        acc[cur ^ 1][2 * lane + 1] = im;
       }
       __syncwarp();
       cur ^= 1;
     }
     if (lane < 16) {  // packed entry (re, re, -im, im)
-      const float re = (float)acc[w][cur][2 * lane], im = (float)acc[w][cur][2 * lane + 1];
+      const float re = (float)acc[cur][2 * lane], im = (float)acc[cur][2 * lane + 1];
       dst[2 * lane] = make_float2(re, re);
       dst[2 * lane + 1] = make_float2(-im, im);
     }
@@ -106,6 +158,14 @@ __global__ void __launch_bounds__(32 * kMatWarps) k_materialize(const MatSlot *_
   }
   const int n_reg = n_slots - n_fused_slots;
   if (n_reg == 0) return;
+  if (spread) {
+    const long long t = (gw - n_fw) * 8 + (lane >> 2);
+    const bool live = t < (long long)n_reg * batch;
+    const int b = live ? (int)(t / n_reg) : 0;
+    materialize_spread(slots[n_fused_slots + (live ? t % n_reg : 0)], params ? params + (long long)b * n_params : nullptr,
+                       out + (long long)b * mstride, lane, live);
+    return;
+  }
   const long long t = (gw - n_fw) * 32 + lane;
   if (t >= (long long)n_reg * batch) return;
   const int b = (int)(t / n_reg);
@@ -117,11 +177,11 @@ cudaError_t launch_materialize(const MatSlot *d_slots, int n_slots, int n_fused_
                                const double *params, int n_params, int batch, long long mstride, float2 *out,
                                cudaStream_t s) {
   const long long nf = (long long)n_fused_slots * batch, nr = (long long)(n_slots - n_fused_slots) * batch;
-  const int per_thread = nf >= kFusedPerThread ? 1 : 0;
-  const long long warps = (per_thread ? (nf + 31) / 32 : nf) + (nr + 31) / 32;
+  const int per_thread = nf >= kFusedPerThread ? 1 : 0, spread = !per_thread && nr <= kSpreadSlots ? 1 : 0;
+  const long long warps = (per_thread ? (nf + 31) / 32 : nf) + (spread ? (nr + 7) / 8 : (nr + 31) / 32);
   if (warps == 0) return cudaSuccess;
-  k_materialize<<<(unsigned)((warps + kMatWarps - 1) / kMatWarps), 32 * kMatWarps, 0, s>>>(
-      d_slots, n_slots, n_fused_slots, d_fused, params, n_params, batch, mstride, out, per_thread);
+  k_materialize<<<(unsigned)warps, 32, 0, s>>>(d_slots, n_slots, n_fused_slots, d_fused, params, n_params, batch, mstride,
+                                               out, per_thread, spread);
   return cudaGetLastError();
 }
 

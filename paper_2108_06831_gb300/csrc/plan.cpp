@@ -572,7 +572,8 @@ tn_status build_pass_plan(const tn_circuit &c, int T, int K, bool adjoint, std::
           const GateCls &gq = P.cls[g];
           const TnGate &tq = c.gates[g];
           const bool hg = adjoint && tq.param_idx >= 0;
-          const int cost = op_code_cost(gq.type, tq.kind, adjoint, hg, hg ? gate_arity(tq.kind) : 0);
+          int cost = op_code_cost(gq.type, tq.kind, adjoint, hg, hg ? gate_arity(tq.kind) : 0);
+          if (Kp < 4 && nS >= kLowBits + 2) cost = std::max(1, cost >> (4 - Kp));  // the costs are of 16 amplitudes
           if (pass_code > 0 && pass_code + cost > kPassCodeBudget) pass_full = true;
           else pass_code += cost;
         }

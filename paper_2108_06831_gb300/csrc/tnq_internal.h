@@ -23,6 +23,18 @@ constexpr int kMaxQubits = 34;   // 2^34 complex64 = 128 GiB, the largest state 
 constexpr int kMaxTile = 13;     // qubits per on-chip tile (2^13 complex64 = 64 KiB of shared memory)
 constexpr int kLowBits = 4;      // the lowest bits always inside a tile: runs of 16 amplitudes = 128 B
 constexpr int kMaxReg = 4;       // register qubits per thread and phase (2^4 amplitudes)
+// Small states: with 16 amplitudes a thread they give an SM too few warps to hide a pass's latency (every
+// gate is a chain of dependent instructions, every phase a barrier).  Below kLeanWarps warps per SM the
+// forward passes run from a plan of kLeanReg register qubits (four amplitudes a thread; one qubit more
+// for states of several tiles): more phases, but four times the warps and a quarter of the instructions
+// in each thread's way.  Below kLeanGates gates that mix amplitudes there is nothing to shorten.  From
+// kFuseMinQubitsParam qubits on a parameterised circuit's 4x4 blocks are read from shared memory by
+// twice the threads, which costs more than the warps gain (16 qubits, 8 sets: 47 against 55 us).
+// Measured: 9 qubits depth 6, one set 20.6 -> 10.4 us; 10 qubits depth 8, 128 sets 26.7 -> 14.4 us.
+constexpr int kConstMinQubits = 19;  // parameterised circuits, batch 1: constant tables from this width on
+constexpr double kLeanWarps = 8.0;
+constexpr double kLeanGates = 24.0;
+constexpr int kLeanReg = 2;
 constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pass of the adjoint sweep
 
 // ---------------------------------------------------------------------------------------
@@ -175,7 +187,19 @@ TNQ_HD int gate_nqubits(int kind) {
           kind == TN_GATE_MAT2 || kind == KIND_F2) ? 2 : 1;
 }
 
-TNQ_HD int gate_matrix(int kind, int form, const double *ang, const double *fixed, double *o) {
+// Arguments of the sines and cosines a kind's matrix is made of; returns their number.
+TNQ_HD int gate_trig(int kind, const double *ang, double *x) {
+  switch (kind) {
+    case TN_GATE_RX: case TN_GATE_RY: case TN_GATE_RZ: x[0] = ang[0] * 0.5; return 1;
+    case TN_GATE_U3: x[0] = ang[0] * 0.5; x[1] = ang[1]; x[2] = ang[2]; return 3;
+    case KIND_V: x[0] = ang[0] * 0.5; x[1] = ang[1]; return 2;
+    case TN_GATE_CP: case KIND_P: x[0] = ang[0]; return 1;
+    default: return 0;
+  }
+}
+
+// The matrix from the sines and cosines of those arguments (which different threads may have evaluated).
+TNQ_HD int gate_matrix_sc(int kind, int form, const double *sn, const double *cs, const double *fixed, double *o) {
   const double r2 = 0.70710678118654752440;
   int dim = gate_nqubits(kind) == 2 ? 4 : 2;
   for (int i = 0; i < 2 * dim * dim; ++i) o[i] = 0.0;
@@ -197,31 +221,25 @@ TNQ_HD int gate_matrix(int kind, int form, const double *ang, const double *fixe
     case TN_GATE_SW:  // cos(pi/4) I - i sin(pi/4) (X+Y)/sqrt2
       cset(o, 0, r2, 0); cset(o, 1, -0.5, -0.5); cset(o, 2, 0.5, -0.5); cset(o, 3, r2, 0); break;
     case TN_GATE_RX: {
-      double c, s;
-      sincos2(ang[0] * 0.5, &s, &c);
+      const double c = cs[0], s = sn[0];
       if (!deriv) { cset(o, 0, c, 0); cset(o, 1, 0, -s); cset(o, 2, 0, -s); cset(o, 3, c, 0); }
       else { cset(o, 0, -0.5 * s, 0); cset(o, 1, 0, -0.5 * c); cset(o, 2, 0, -0.5 * c); cset(o, 3, -0.5 * s, 0); }
       break;
     }
     case TN_GATE_RY: {
-      double c, s;
-      sincos2(ang[0] * 0.5, &s, &c);
+      const double c = cs[0], s = sn[0];
       if (!deriv) { cset(o, 0, c, 0); cset(o, 1, -s, 0); cset(o, 2, s, 0); cset(o, 3, c, 0); }
       else { cset(o, 0, -0.5 * s, 0); cset(o, 1, -0.5 * c, 0); cset(o, 2, 0.5 * c, 0); cset(o, 3, -0.5 * s, 0); }
       break;
     }
     case TN_GATE_RZ: {
-      double c, s;
-      sincos2(ang[0] * 0.5, &s, &c);
+      const double c = cs[0], s = sn[0];
       if (!deriv) { cset(o, 0, c, -s); cset(o, 3, c, s); }
       else { cset(o, 0, -0.5 * s, -0.5 * c); cset(o, 3, -0.5 * s, 0.5 * c); }
       break;
     }
     case TN_GATE_U3: {
-      double c, s, cp, sp, cl, sl;
-      sincos2(ang[0] * 0.5, &s, &c);
-      sincos2(ang[1], &sp, &cp);
-      sincos2(ang[2], &sl, &cl);
+      const double c = cs[0], s = sn[0], cp = cs[1], sp = sn[1], cl = cs[2], sl = sn[2];
       const double cpl = cp * cl - sp * sl, spl = sp * cl + cp * sl;  // e^{i(p+l)}
       if (!deriv) {
         cset(o, 0, c, 0); cset(o, 1, -cl * s, -sl * s); cset(o, 2, cp * s, sp * s); cset(o, 3, cpl * c, spl * c);
@@ -238,8 +256,7 @@ TNQ_HD int gate_matrix(int kind, int form, const double *ang, const double *fixe
     case TN_GATE_CZ: cset(o, 0, 1, 0); cset(o, 5, 1, 0); cset(o, 10, 1, 0); cset(o, 15, -1, 0); break;
     case TN_GATE_CNOT: cset(o, 0, 1, 0); cset(o, 5, 1, 0); cset(o, 11, 1, 0); cset(o, 14, 1, 0); break;
     case TN_GATE_CP: {
-      double c, s;
-      sincos2(ang[0], &s, &c);
+      const double c = cs[0], s = sn[0];
       if (!deriv) { cset(o, 0, 1, 0); cset(o, 5, 1, 0); cset(o, 10, 1, 0); cset(o, 15, c, s); }
       else { cset(o, 15, -s, c); }
       break;
@@ -247,15 +264,12 @@ TNQ_HD int gate_matrix(int kind, int form, const double *ang, const double *fixe
     case TN_GATE_SWAP: cset(o, 0, 1, 0); cset(o, 6, 1, 0); cset(o, 9, 1, 0); cset(o, 15, 1, 0); break;
     case TN_GATE_MAT1: for (int i = 0; i < 8; ++i) o[i] = fixed[i]; break;
     case KIND_V: {
-      double c, s, ca, sa;
-      sincos2(ang[0] * 0.5, &s, &c);
-      sincos2(ang[1], &sa, &ca);
+      const double c = cs[0], s = sn[0], ca = cs[1], sa = sn[1];
       cset(o, 0, c, 0); cset(o, 1, -s * ca, -s * sa); cset(o, 2, s, 0); cset(o, 3, c * ca, c * sa);
       break;
     }
     case KIND_P: {
-      double c, s;
-      sincos2(ang[0], &s, &c);
+      const double c = cs[0], s = sn[0];
       cset(o, 0, 1, 0);
       cset(o, 3, c, s);
       break;
@@ -266,6 +280,13 @@ TNQ_HD int gate_matrix(int kind, int form, const double *ang, const double *fixe
   return dim;
 }
 
+TNQ_HD int gate_matrix(int kind, int form, const double *ang, const double *fixed, double *o) {
+  double x[3] = {0.0, 0.0, 0.0}, sn[3] = {0.0, 0.0, 0.0}, cs[3] = {0.0, 0.0, 0.0};
+  const int n = gate_trig(kind, ang, x);
+  for (int a = 0; a < n; ++a) sincos2(x[a], &sn[a], &cs[a]);
+  return gate_matrix_sc(kind, form, sn, cs, fixed, o);
+}
+
 // Number of angles a kind reads.
 TNQ_HD int gate_arity(int kind) {
   return kind == TN_GATE_U3 ? 3 : kind == KIND_V ? 2
@@ -274,9 +295,9 @@ TNQ_HD int gate_arity(int kind) {
 
 // Entries of a matrix slot: the full matrix in the shape the op consumes, optionally
 // conjugate-transposed (FORM_ADJ).  Writes complex64 (float2) entries to dst.
-TNQ_HD int slot_entries(const MatSlot &s, const double *ang, double *tmp /*32*/, float *dst) {
+TNQ_HD int slot_entries(const MatSlot &s, const double *sn, const double *cs, double *tmp /*32*/, float *dst) {
   int form = s.form == FORM_ADJ ? FORM_U : s.form;
-  int dim = gate_matrix(s.kind, form, ang, s.fixed, tmp);
+  int dim = gate_matrix_sc(s.kind, form, sn, cs, s.fixed, tmp);
   bool adj = s.form == FORM_ADJ;
   auto put = [&](int k, int i, int j) {  // dst entry k <- (adj ? conj(m[j][i]) : m[i][j])
     int src = adj ? (j * dim + i) : (i * dim + j);
@@ -359,13 +380,10 @@ TNQ_HD void fused_apply_member(const FusedMember &f, const double *param_row, do
 }
 
 // One member of a fused block as a 4x4 on (a, b), indexed 2 bit(a) + bit(b), FP64 (re, im) pairs.
-TNQ_HD void fused_embed(const FusedMember &f, const double *param_row, double *e /*32*/) {
-  double ang[3] = {f.angle[0], f.angle[1], f.angle[2]};
-  for (int a = 0; a < 3; ++a)
-    for (int k = 0; k < 2; ++k)
-      if (f.pidx[a][k] >= 0 && param_row) ang[a] += param_row[f.pidx[a][k]];
+// sn, cs: the sines and cosines of gate_trig's arguments.
+TNQ_HD void fused_embed(const FusedMember &f, const double *sn, const double *cs, double *e /*32*/) {
   double g[32];
-  const int dim = gate_matrix(f.kind, FORM_U, ang, f.mat, g);
+  const int dim = gate_matrix_sc(f.kind, FORM_U, sn, cs, f.mat, g);
   for (int i = 0; i < 4; ++i)
     for (int j = 0; j < 4; ++j) {
       const int ia = i >> 1, ib = i & 1, ja = j >> 1, jb = j & 1;
@@ -448,6 +466,8 @@ struct tn_plan {
   int n_params;
   uint64_t init;
   int T, K;
+  tn_plan *lean = nullptr;  // plan of the same circuit that runs the forward passes instead (few warps), or NULL
+  bool is_lean = false;
   tn_plan_opts opts;
   bool host_only;
   int device;

@@ -229,3 +229,25 @@ def test_tile_autotuner_single_plan():
         assert rel_l2(got[b], simulate_state(c, params[b])) <= STATE_TOL
     with pytest.raises(tn.TnError):  # tile_qubits is the tuner's choice
         tn.Plan(tn.CircuitHandle(c), tile_qubits=10, tune={})
+
+
+@pytest.mark.parametrize("n,depth,batch,parameterized", [
+    (6, 5, 3, True), (8, 4, 1215, True), (9, 3, 1216, True), (12, 6, 2, True), (13, 4, 3, True), (14, 4, 2, True),
+    (6, 8, 1, False), (12, 8, 1, False), (13, 6, 1, False), (16, 5, 1, False), (18, 4, 1, False)])
+def test_small_states_take_few_amplitudes_per_thread(n, depth, batch, parameterized):
+    """Plans of few warps run four (or eight) amplitudes per thread: one tile and several, either side of the
+    rule's limits, tables staged and constant, the gate tables of few and of many slots; as amplitudes too."""
+    from oracle.statevector import simulate_state
+    tn = _tn()
+    c, _ = C.brickwork(n, depth, 50 + n, parameterized=parameterized)
+    c.init_basis = (n * 977) % (1 << n)
+    params = np.random.default_rng(n).uniform(0, 2 * np.pi, size=(batch, c.n_params)) if parameterized else None
+    got = gpu_state(c, params, batch=batch)
+    xs = np.arange(0, 1 << n, 37)
+    ctr = tn.Contractor(c, target=tn.TARGET_AMPLITUDES, batch=batch)
+    p = None if params is None else torch.as_tensor(params, device="cuda")
+    amps = ctr.amplitudes(torch.as_tensor(xs, device="cuda"), p).cpu().numpy()
+    for b in sorted({0, batch // 2, batch - 1}):
+        ref = simulate_state(c, None if params is None else params[b])
+        assert rel_l2(got[b], ref) <= STATE_TOL
+        assert rel_l2(amps[b], ref[xs]) <= STATE_TOL
