@@ -1,5 +1,6 @@
 // C ABI of libtnq (declared in include/tn.h): argument checks, plan construction and
 // upload, workspace layout, and the launch sequences of the contraction calls.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdlib>
 #include <cstdio>
@@ -55,6 +56,19 @@ int num_sms() {
     g_sms.count[dev] = v > 0 ? v : 1;
   }
   return g_sms.count[dev];
+}
+
+long long grid_per_row(long long n_tiles, long long batch, int per_sm) {
+  const long long slots = (long long)num_sms() * std::max(per_sm, 1);
+  const long long most = std::max<long long>(1, std::min(n_tiles, (4 * slots + batch - 1) / batch));
+  long long best = 1;
+  double best_cost = 0.0;
+  for (long long gx = 1; gx <= most; ++gx) {
+    // tiles of a CTA, and one more for its start and end, times the waves
+    const double cost = (double)((n_tiles + gx - 1) / gx + 1) * (double)((gx * batch + slots - 1) / slots);
+    if (gx == 1 || cost < best_cost) best = gx, best_cost = cost;
+  }
+  return best;
 }
 
 // The dynamic shared-memory limit of a kernel is a per-device function attribute: raise it on

@@ -220,9 +220,7 @@ cudaError_t launch_bwd_k(const PassDesc &h, const PassDesc *d_pass, const tn_pla
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   const long long n_tiles = 1ll << h.n_outer;
-  long long gx = ((long long)num_sms() * per_sm + p->batch - 1) / p->batch;
-  if (gx > n_tiles) gx = n_tiles;
-  if (gx < 1) gx = 1;
+  const long long gx = grid_per_row(n_tiles, p->batch, per_sm);
   dim3 grid((unsigned)gx, (unsigned)p->batch);
   k_bwd_pass<K><<<grid, threads, smem, s>>>(d_pass, p->d_bwd_phase, p->d_bwd_ops, p->d_bwd_grads, mats, mstride, psi,
                                             lam, grad, p->n_params, p->n);
@@ -240,9 +238,7 @@ cudaError_t launch_backward(const tn_plan *p, const float2 *mats, long long mstr
       const int per_sm = i < p->jit_bwd_grid.size() ? p->jit_bwd_grid[i] : 1;  // queried at load time
       cudaError_t e = cudaSuccess;
       const long long n_tiles = 1ll << h.n_outer;
-      long long gx = ((long long)num_sms() * per_sm + p->batch - 1) / p->batch;
-      if (gx > n_tiles) gx = n_tiles;
-      if (gx < 1) gx = 1;
+      const long long gx = grid_per_row(n_tiles, p->batch, per_sm);
       const float2 *m = mats;
       int np = p->n_params;
       void *args[] = {(void *)&m, (void *)&mstride, (void *)&psi, (void *)&lam, (void *)&grad, (void *)&np};

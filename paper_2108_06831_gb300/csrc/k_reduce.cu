@@ -431,12 +431,7 @@ int red_grid_x(const tn_observable *o, int pass, int batch) {
   const RedPass &rp = o->passes[pass];
   const long long per_sm =
       std::max<long long>(1, std::min<long long>(kRedCtas, (227 * 1024) / (long long)(red_smem(rp) + 2048)));
-  long long gx = ((long long)num_sms() * per_sm + batch - 1) / batch;
-  const long long n_tiles = 1ll << rp.n_outer;
-  if (gx > n_tiles) gx = n_tiles;
-  if (gx > kRedMaxCTAs) gx = kRedMaxCTAs;
-  if (gx < 1) gx = 1;
-  return (int)gx;
+  return (int)std::min<long long>(kRedMaxCTAs, grid_per_row(1ll << rp.n_outer, batch, (int)per_sm));
 }
 }  // namespace
 

@@ -8,6 +8,10 @@
 namespace tnq {
 
 int num_sms();  // SM count of the current device (cached per device)
+// Grid width of a kernel whose `batch` rows of CTAs each stride over n_tiles tiles, per_sm of them
+// resident per SM.  Rows of ceil(slots / batch) CTAs would leave a few CTAs for a second wave that lasts
+// as long as the first (64 rows of 10 on 608 slots).
+long long grid_per_row(long long n_tiles, long long batch, int per_sm);
 
 #ifdef __CUDACC__
 // Programmatic dependent launch (short kernels of the network path).  A kernel launched with
