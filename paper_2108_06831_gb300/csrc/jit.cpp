@@ -559,9 +559,10 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
 // application and a dot.
 bool pauli_rotation(int kind) { return kind == TN_GATE_RX || kind == TN_GATE_RY || kind == TN_GATE_RZ; }
 
-void emit_grad_pauli(Emitter &E, const OpDesc &op, int kind, const GradRec &gr, int nwarps) {
+void emit_grad_pauli(Emitter &E, const OpDesc &op, int kind, const std::string &var) {
   const int R = E.R;
   char buf[320];
+  E.line("float " + var + ";");
   E.line("{ float acc = 0.f;");
   if (kind == TN_GATE_RZ) {  // Im <l|Z|a> = sum_j (-1)^{bit_j} (l.x a.y - l.y a.x)
     const bool reg = op.a_kind == SRC_REG;
@@ -590,17 +591,13 @@ void emit_grad_pauli(Emitter &E, const OpDesc &op, int kind, const GradRec &gr, 
       E.line(buf);
     }
   }
-  E.line("  acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 16); acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 8);");
-  E.line("  acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 4); acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 2);");
-  E.line("  acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 1);");
-  snprintf(buf, sizeof buf, "  if (lane == 0) wacc[%d + warp] += acc;", gr.slot * nwarps);
-  E.line(buf);
-  E.line("}");
+  E.line("  " + var + " = acc; }");
 }
 
-void emit_grad(Emitter &E, const OpDesc &op, int kind, const GradRec &gr, int nwarps) {
+void emit_grad(Emitter &E, const OpDesc &op, int kind, const GradRec &gr, const std::string &var) {
   const int R = E.R;
   char buf[320];
+  E.line("float " + var + ";");
   auto mat = [&](int k) {
     snprintf(buf, sizeof buf, "f2(M4[%d], %d)", (gr.mat + k) >> 1, (gr.mat + k) & 1);
     return std::string(buf);
@@ -674,12 +671,47 @@ void emit_grad(Emitter &E, const OpDesc &op, int kind, const GradRec &gr, int nw
     if (!cond.empty()) E.line("  }");
   }
   E.line("  acc = 2.f * acc;");
-  E.line("  acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 16); acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 8);");
-  E.line("  acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 4); acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 2);");
-  E.line("  acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 1);");
-  snprintf(buf, sizeof buf, "  if (lane == 0) wacc[%d + warp] += acc;", gr.slot * nwarps);
-  E.line(buf);
+  E.line("  " + var + " = acc; }");
+}
+
+// Warp sums of up to four pending dots (phase variables and their slots), added to the pass's accumulation
+// slots.  One dot takes five butterfly steps; two or four share the first steps, in which half of the
+// lanes go on with one dot and half with the other (6 shuffles for four dots instead of 20).  Every dot is
+// summed in the same tree: lanes 16 apart first, then 8, 4, 2, 1.
+struct PendingDot {
+  std::string var;
+  int slot;
+};
+void emit_dot_sums(Emitter &E, std::vector<PendingDot> &dots, int nwarps) {
+  const size_t n = dots.size();
+  if (n == 0) return;
+  auto v = [&](size_t i) { return i < n ? dots[i].var : std::string("0.f"); };
+  // the two dots x and y over lane bit b: x where the bit is 0, y where it is 1
+  auto merge = [&](const std::string &out, const std::string &x, const std::string &y, int b) {
+    const std::string B = std::to_string(b);
+    E.line("  float " + out + " = (lane & " + B + ") ? " + y + " : " + x + "; { const float t = (lane & " + B + ") ? " + x +
+           " : " + y + "; " + out + " += __shfl_xor_sync(0xFFFFFFFFu, t, " + B + "); }");
+  };
+  E.line("{");
+  int last = 16;  // the next butterfly step
+  if (n == 1) {
+    E.line("  float r = " + v(0) + ";");
+  } else if (n == 2) {
+    merge("r", v(0), v(1), 16);
+    last = 8;
+  } else {
+    merge("r01", v(0), v(1), 16);
+    merge("r23", v(2), v(3), 16);
+    merge("r", "r01", "r23", 8);
+    last = 4;
+  }
+  for (int b = last; b > 0; b >>= 1) E.line("  r += __shfl_xor_sync(0xFFFFFFFFu, r, " + std::to_string(b) + ");");
+  // dot 0 is complete on lane 0, 1 on lane 16, 2 on lane 8, 3 on lane 24
+  const int home[4] = {0, 16, 8, 24};
+  for (size_t i = 0; i < n; ++i)
+    E.line("  if (lane == " + std::to_string(home[i]) + ") wacc[" + std::to_string(dots[i].slot * nwarps) + " + warp] += r;");
   E.line("}");
+  dots.clear();
 }
 
 std::string rename_array(const std::string &code, const char *to) {
@@ -810,6 +842,23 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
   E.line("    asm volatile(\"cp.async.commit_group;\" ::: \"memory\");");
   E.line("    asm volatile(\"cp.async.wait_group 0;\" ::: \"memory\");");
   E.line("    __syncthreads();");
+  // the next tile on its way to L2 while this one is computed
+  E.line("    if (t + gridDim.x < " + std::to_string(NT) + "ll) {");
+  E.line("      const long long t2 = t + gridDim.x; " + emit_base("t2", "base2"));
+  // one prefetch per 128-byte run (16 amplitudes)
+  {
+    std::string dep = "0ll";
+    for (int j = 0; j < T - 4; ++j) {
+      snprintf(buf, sizeof buf, " | ((long long)((run >> %d) & 1) << %d)", j, (int)pd.tile_pos[4 + j]);
+      dep += buf;
+    }
+    snprintf(buf, sizeof buf, "      for (int run = tid; run < %d; run += %d) {", 1 << (T - 4), NTHR);
+    E.line(buf);
+    E.line("        const long long at = base2 + (" + dep + ");");
+    E.line("        asm volatile(\"prefetch.global.L2 [%0];\" :: \"l\"(gp + at)); asm volatile(\"prefetch.global.L2 [%0];\" :: \"l\"(gl + at));");
+    E.line("      }");
+  }
+  E.line("    }");
   for (int ph = pd.phase_begin; ph < pd.phase_end; ++ph) {
     const PhaseDesc &d = p.bwd.phases[ph];
     E.line("    {");
@@ -830,8 +879,14 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
       snprintf(buf, sizeof buf, "      a[%d] = smp[pb ^ %d]; l[%d] = sml[pb ^ %d];", j, ro[j], j, ro[j]);
       E.line(buf);
     }
+    std::vector<PendingDot> dots;
+    auto pend = [&](const GradRec &gr) {
+      dots.push_back({"dot" + std::to_string(gr.slot), gr.slot});
+      return dots.back().var;
+    };
     for (int o = d.op_begin; o < d.op_end; ++o) {
       const OpDesc &op = p.bwd.ops[o];
+      if (dots.size() + op.n_grad > 4) emit_dot_sums(E, dots, NW);
       Emitter tmp;
       tmp.K = K;
       tmp.R = E.R;
@@ -839,12 +894,16 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
       const std::string code_a = tmp.o.str();
       const bool pauli = op.has_grad && pauli_rotation(op_kind[o]);
       if (pauli)  // from psi_k, lambda_k
-        for (int g = 0; g < op.n_grad; ++g) emit_grad_pauli(E, op, op_kind[o], p.bwd.grads[(size_t)(op.aux + g)], NW);
+        for (int g = 0; g < op.n_grad; ++g) emit_grad_pauli(E, op, op_kind[o], pend(p.bwd.grads[(size_t)(op.aux + g)]));
       E.o << code_a;  // psi_{k-1} = U^dag psi_k
       if (op.has_grad && !pauli)
-        for (int g = 0; g < op.n_grad; ++g) emit_grad(E, op, op_kind[o], p.bwd.grads[(size_t)(op.aux + g)], NW);
+        for (int g = 0; g < op.n_grad; ++g) {
+          const GradRec &gr = p.bwd.grads[(size_t)(op.aux + g)];
+          emit_grad(E, op, op_kind[o], gr, pend(gr));
+        }
       E.o << rename_array(code_a, "l");  // lambda_{k-1} = U^dag lambda_k
     }
+    emit_dot_sums(E, dots, NW);
     for (int j = 0; j < E.R; ++j) {
       snprintf(buf, sizeof buf, "      smp[pb ^ %d] = a[%d]; sml[pb ^ %d] = l[%d];", ro[j], j, ro[j], j);
       E.line(buf);
