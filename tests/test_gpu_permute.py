@@ -75,3 +75,23 @@ def test_rejects_bad_perm():
         tn.permute(4, [0, 1, 1, 2], 1, x, y)
     with pytest.raises(tn.TnError):
         tn.permute(4, [0, 1, 2, 3], 1, x, x)
+
+
+@pytest.mark.parametrize("n", [5, 6, 7, 9, 11, 12, 13])
+def test_tiles_of_every_row_count(n):
+    """Around the tile's size: direct mapping, one row, fewer rows than a tile holds, one tile and two; from
+    no low leg moved to all of them."""
+    rng = np.random.default_rng(n)
+    from paper_2108_06831_gb300 import tn
+    batch = 3
+    x = (rng.normal(size=(batch, 1 << n)) + 1j * rng.normal(size=(batch, 1 << n))).astype(np.complex64)
+    perms = [list(range(n)), list(range(n))[::-1], list(np.roll(range(n), 1)), list(np.roll(range(n), n // 2))]
+    perms += [rng.permutation(n) for _ in range(6)]
+    xin = torch.as_tensor(x, device="cuda")
+    for perm in perms:
+        perm = [int(v) for v in perm]
+        out = torch.empty_like(xin)
+        tn.permute(n, perm, batch, xin, out)
+        torch.cuda.synchronize()
+        assert tn.sync_status() == tn.OK
+        assert np.array_equal(out.cpu().numpy(), _ref(x, n, perm))
