@@ -54,6 +54,10 @@ constexpr int kColBits = 6;  // log2 of the complex columns of a tile (BN / 2)
 static_assert(BN / 2 == 1 << kColBits, "column table covers one tile");
 constexpr int kMain = 3;                      // leading-product accumulators, used round robin by K tile
 constexpr int kTmemCols = (kMain + 1) * BN;   // + one correction accumulator = all 512 columns
+// tensor-memory columns of k_cgemm_tc's accumulators: the correction one between the first two leading
+// ones, so that it is adjacent to either
+constexpr int kCorrCol = BN;
+__host__ __device__ constexpr int lead_col(int j) { return j == 0 ? 0 : (j + 1) * BN; }
 constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of every mbarrier wait
 constexpr int kRasterRows = 8;  // row tiles per group of the tile order (k_cgemm_tc)
 
@@ -292,8 +296,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgemm_tc(const __grid_constant_
         const int kc = kt * (KBYTES / CF::kElem);
         const int a_loads = SPLIT_A ? 1 : CF::kParts;
         for (int p = 0; p < a_loads; ++p) tma_load_3d(st + p * kTileA, &maps.a[p], &full[s], kc, m0, bz);
-        for (int p = 0; p < CF::kParts; ++p)
-          tma_load_3d(st + CF::kParts * kTileA + p * kTileB, &maps.b[p], &full[s], kc, n0, bz);
+        for (int p = 0; p < CF::kParts; ++p) {
+          const int at = kt % kMain == 1 && p < 2 ? 1 - p : p;  // see the MMA issuer
+          tma_load_3d(st + CF::kParts * kTileA + at * kTileB, &maps.b[p], &full[s], kc, n0, bz);
+        }
       }
     }
   } else if (warp == 5) {
@@ -308,21 +314,35 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgemm_tc(const __grid_constant_
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t st = saddr(smem + (size_t)s * stage_bytes);
+        // product 0 (the leading parts) of K tile kt accumulates in lead_col(j), j = kt mod kMain; the
+        // correction products in kCorrCol.  Small terms never meet the large running sum inside the
+        // MMA, and each leading accumulator sees a third of the K steps.  Products 0 and 1 share A's
+        // leading part; for j = 0 and 1 their accumulators are adjacent, and B's first two parts lie in
+        // the accumulators' order (leading, correction; for j = 1 correction, leading): one MMA of 2 BN
+        // columns does both and reads A once.  The sums keep their order.
+        constexpr int kSteps = KBYTES / (CF::kMmaK * CF::kElem);
+        const int j = kt % kMain;
+        const uint32_t b_at = st + CF::kParts * kTileA;
+        const uint32_t b_lead = b_at + (j == 1 ? kTileB : 0), b_corr = b_at + (j == 1 ? 0 : kTileB);
 #pragma unroll
-        for (int p = 0; p < CF::kProducts; ++p) {
+        for (int kk = 0; kk < kSteps; ++kk) {
+          const uint32_t off = kk * CF::kMmaK * CF::kElem;  // 32 bytes per MMA along K
+          const bool acc_lead = kt >= kMain || kk > 0, acc_corr = kt > 0 || kk > 0;
+          if (j < 2 && acc_lead == acc_corr) {
+            mma<PREC, 2 * BN>(tmem_d + (uint32_t)(j * BN), smem_desc(st + off), smem_desc(b_at + off), acc_lead ? 1u : 0u);
+          } else {
+            mma<PREC>(tmem_d + (uint32_t)lead_col(j), smem_desc(st + off), smem_desc(b_lead + off), acc_lead ? 1u : 0u);
+            mma<PREC>(tmem_d + kCorrCol, smem_desc(st + off), smem_desc(b_corr + off), acc_corr ? 1u : 0u);
+          }
+        }
+#pragma unroll
+        for (int p = 2; p < CF::kProducts; ++p) {
           const uint32_t a_base = st + CF::pa(p) * kTileA;
-          const uint32_t b_base = st + CF::kParts * kTileA + CF::pb(p) * kTileB;
+          const uint32_t b_base = CF::pb(p) == 0 ? b_lead : CF::pb(p) == 1 ? b_corr : b_at + CF::pb(p) * kTileB;
 #pragma unroll
-          for (int kk = 0; kk < KBYTES / (CF::kMmaK * CF::kElem); ++kk) {
-            const uint32_t off = kk * CF::kMmaK * CF::kElem;  // 32 bytes per MMA along K
-            // product 0 (the leading parts) of K tile kt accumulates in columns [j BN, (j+1) BN),
-            // j = kt mod kMain; the correction products in [kMain BN, (kMain+1) BN).  Small terms
-            // never meet the large running sum inside the MMA, and each leading accumulator sees
-            // a third of the K steps.
-            const int j = kt % kMain;
-            const uint32_t dst = tmem_d + (uint32_t)((p == 0 ? j : kMain) * BN);
-            const bool acc = p == 0 ? (kt >= kMain || kk > 0) : (kt > 0 || kk > 0 || p > 1);
-            mma<PREC>(dst, smem_desc(a_base + off), smem_desc(b_base + off), acc ? 1u : 0u);
+          for (int kk = 0; kk < kSteps; ++kk) {
+            const uint32_t off = kk * CF::kMmaK * CF::kElem;
+            mma<PREC>(tmem_d + kCorrCol, smem_desc(a_base + off), smem_desc(b_base + off), 1u);
           }
         }
         mma_issued = true;
@@ -373,14 +393,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgemm_tc(const __grid_constant_
       float v[32];
       {
         uint32_t e[32];
-        tmem_ld32(taddr + kMain * BN, e);
+        tmem_ld32(taddr + kCorrCol, e);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(e[i]);
       }
       for (int j = 0; j < n_main; ++j) {  // corrections first, then the leading sums in order
         uint32_t r[32];
-        tmem_ld32(taddr + j * BN, r);
+        tmem_ld32(taddr + lead_col(j), r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] += __uint_as_float(r[i]);
@@ -770,62 +790,63 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N) {
 
 // ------------------------------------------------------------------------------ prep kernels
 
-// A (real view [rows][cols]) -> parts
+// The parts of four consecutive elements, 16 (TF32) or 8 (BF16) bytes of each part per thread.
+template <int PREC>
+__device__ __forceinline__ void store_parts(float4 v, long long at, void *p0, void *p1, void *p2) {
+  if constexpr (PREC == PREC_TF32) {
+    const float4 h = make_float4(tf32_rna(v.x), tf32_rna(v.y), tf32_rna(v.z), tf32_rna(v.w));
+    *reinterpret_cast<float4 *>(static_cast<float *>(p0) + at) = h;
+    *reinterpret_cast<float4 *>(static_cast<float *>(p1) + at) = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+  } else {
+    const float x[4] = {v.x, v.y, v.z, v.w};
+    uint32_t w[3][2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      uint32_t h[3][2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const __nv_bfloat16 b0 = __float2bfloat16_rn(x[2 * q + e]);
+        const float r1 = x[2 * q + e] - __bfloat162float(b0);
+        const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
+        h[0][e] = __bfloat16_as_ushort(b0);
+        h[1][e] = __bfloat16_as_ushort(b1);
+        h[2][e] = __bfloat16_as_ushort(__float2bfloat16_rn(r1 - __bfloat162float(b1)));
+      }
+#pragma unroll
+      for (int p = 0; p < 3; ++p) w[p][q] = h[p][0] | (h[p][1] << 16);
+    }
+    void *const part[3] = {p0, p1, p2};
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+      *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(part[p]) + at) = make_uint2(w[p][0], w[p][1]);
+  }
+}
+
+// A (n real values, a multiple of 4: operand rows are multiples of 16 bytes) -> parts.  HBM-bound: 4096 x
+// 4096 complex into TF32 parts 98 us with one element per thread and store, 66 with four.
 template <int PREC>
 __global__ void k_split(const float *__restrict__ x, long long n, void *p0, void *p1, void *p2) {
   pdl_wait();
   pdl_trigger();
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float v = x[i];
-    if constexpr (PREC == PREC_TF32) {
-      const float hi = tf32_rna(v);
-      static_cast<float *>(p0)[i] = hi;
-      static_cast<float *>(p1)[i] = v - hi;
-    } else {
-      const __nv_bfloat16 b0 = __float2bfloat16_rn(v);
-      const float r1 = v - __bfloat162float(b0);
-      const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
-      const float r2 = r1 - __bfloat162float(b1);
-      static_cast<__nv_bfloat16 *>(p0)[i] = b0;
-      static_cast<__nv_bfloat16 *>(p1)[i] = b1;
-      static_cast<__nv_bfloat16 *>(p2)[i] = __float2bfloat16_rn(r2);
-    }
-  }
+  for (long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); i < n;
+       i += 4 * (long long)gridDim.x * blockDim.x)
+    store_parts<PREC>(*reinterpret_cast<const float4 *>(x + i), i, p0, p1, p2);
 }
 
-// B (complex [N][K]) -> 2x2 real embedding [2N][2K], then split.
+// B (complex [N][K], K even) -> 2x2 real embedding [2N][2K], then split: two values of k per thread.
 template <int PREC>
 __global__ void k_embed_split(const float2 *__restrict__ b, long long N, long long K, long long batch, void *p0,
                               void *p1, void *p2) {
   pdl_wait();
   pdl_trigger();
-  const long long total = batch * N * K;
+  const long long half = K / 2, total = batch * N * half;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    const long long bb = i / (N * K), r = i % (N * K), n = r / K, k = r % K;
-    const float2 v = b[i];
-    const long long base = bb * (2 * N) * (2 * K);
-    const long long i0 = base + (2 * n) * (2 * K) + 2 * k;      // row 2n:   (re, -im)
-    const long long i1 = base + (2 * n + 1) * (2 * K) + 2 * k;  // row 2n+1: (im,  re)
-    const float e[4] = {v.x, -v.y, v.y, v.x};
-    const long long at[4] = {i0, i0 + 1, i1, i1 + 1};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float x = e[q];
-      if constexpr (PREC == PREC_TF32) {
-        const float hi = tf32_rna(x);
-        static_cast<float *>(p0)[at[q]] = hi;
-        static_cast<float *>(p1)[at[q]] = x - hi;
-      } else {
-        const __nv_bfloat16 b0 = __float2bfloat16_rn(x);
-        const float r1 = x - __bfloat162float(b0);
-        const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
-        const float r2 = r1 - __bfloat162float(b1);
-        static_cast<__nv_bfloat16 *>(p0)[at[q]] = b0;
-        static_cast<__nv_bfloat16 *>(p1)[at[q]] = b1;
-        static_cast<__nv_bfloat16 *>(p2)[at[q]] = __float2bfloat16_rn(r2);
-      }
-    }
+    const long long row = i / half, k = 2 * (i - row * half);  // row = bb N + n
+    const float4 v = reinterpret_cast<const float4 *>(b)[i];
+    const long long at = 4 * row * K + 2 * k;  // rows 2 row: (re, -im), and 2 row + 1: (im, re)
+    store_parts<PREC>(make_float4(v.x, -v.y, v.z, -v.w), at, p0, p1, p2);
+    store_parts<PREC>(make_float4(v.y, v.x, v.w, v.z), at + 2 * K, p0, p1, p2);
   }
 }
 
@@ -902,11 +923,11 @@ cudaError_t run_tc(long long batch, long long M, long long N, long long K, const
     ap[0] = const_cast<float2 *>(A);  // the GEMM reads A itself (FP32) and splits it on chip
   } else {
     const long long na = batch * M * 2 * K;
-    e = launch_pdl(k_split<PREC>, dim3((unsigned)std::min<long long>((na + 255) / 256, 65535)), dim3(256), 0, s,
+    e = launch_pdl(k_split<PREC>, dim3((unsigned)std::min<long long>((na / 4 + 255) / 256, 65535)), dim3(256), 0, s,
                    reinterpret_cast<const float *>(A), na, ap[0], ap[1], ap[2]);
     if (e != cudaSuccess) return e;
   }
-  const long long nb = batch * N * K;
+  const long long nb = batch * N * K / 2;
   e = launch_pdl(k_embed_split<PREC>, dim3((unsigned)std::min<long long>((nb + 255) / 256, 65535)), dim3(256), 0, s,
                  B, N, K, batch, bp[0], bp[1], bp[2]);
   if (e != cudaSuccess) return e;
