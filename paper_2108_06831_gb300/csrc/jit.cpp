@@ -62,6 +62,7 @@ __device__ __forceinline__ float2 cm(float2 a, float2 b) {
   return up(fma2(pk(a.x, a.x), pk(b.x, b.y), mul2(pk(a.y, a.y), pk(-b.y, b.x))));
 }
 __device__ __forceinline__ float2 ng(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sx(float2 a, unsigned s) { return make_float2(__uint_as_float(__float_as_uint(a.x) ^ s), __uint_as_float(__float_as_uint(a.y) ^ s)); }
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return up(add2(pk(a.x, a.y), pk(b.x, b.y))); }
 // r*x + b*y with r real
 __device__ __forceinline__ float2 rc(float r, float2 x, float2 b, float2 y) {
@@ -318,6 +319,89 @@ void emit_op(Emitter &E, const OpDesc &op, int kind) {
   }
 }
 
+// Deferred diagonal ops of one phase (plans other than expectation plans).  A diagonal factor whose
+// condition reads only bits outside the registers is one number per thread: the phases of a run of such
+// ops multiply into a per-thread scalar (their signs into a sign word) and are applied to the
+// amplitudes once, all of them (q4) or those with register bit r set (q<r>), before the next op that
+// mixes bit r or at the end of the phase.  The circuit's own order among them does not matter: diagonal
+// ops commute, and bits outside the registers are not mixed within a phase.  A QFT's ladder of
+// controlled phases then costs each amplitude one multiplication per register qubit instead of one per
+// gate: 22 qubits 74 -> 53 us, 24 qubits 300 -> 197.  Expectation plans keep the op-by-op form, whose FP32 roundings their
+// FP64 energies and gradients show.
+struct Deferred {
+  bool q[5] = {false, false, false, false, false}, q_decl[5] = {false, false, false, false, false};
+  bool s[5] = {false, false, false, false, false}, s_decl[5] = {false, false, false, false, false};
+  static constexpr int kAll = 4;
+
+  void phase(Emitter &E, int r, const std::string &cond, const std::string &e, const std::string &other) {
+    const std::string v = "q" + std::to_string(r);
+    if (!q_decl[r]) E.line("float2 " + v + ";");
+    q_decl[r] = true;
+    if (!q[r]) E.line(v + " = (" + cond + ") ? " + e + " : " + other + ";");
+    else if (other == "make_float2(1.f, 0.f)") E.line("if (" + cond + ") " + v + " = cm(" + v + ", " + e + ");");
+    else E.line(v + " = cm(" + v + ", (" + cond + ") ? " + e + " : " + other + ");");
+    q[r] = true;
+  }
+  void sign(Emitter &E, int r, const std::string &cond) {
+    const std::string v = "g" + std::to_string(r);
+    if (!s_decl[r]) E.line("unsigned " + v + ";");
+    s_decl[r] = true;
+    E.line(v + (s[r] ? " ^= " : " = ") + "(unsigned)(" + cond + ") << 31;");
+    s[r] = true;
+  }
+  // what is pending on register bit r (kAll: on every amplitude), applied to the registers
+  void flush(Emitter &E, int r) {
+    const std::string n = std::to_string(r);
+    for (int j = 0; j < E.R && (q[r] || s[r]); ++j) {
+      if (r != kAll && !(j & (1 << r))) continue;
+      const std::string a = "a[" + std::to_string(j) + "]";
+      std::string v = a;
+      if (s[r]) v = "sx(" + v + ", g" + n + ")";
+      if (q[r]) v = "cm(" + v + ", q" + n + ")";
+      E.line(a + " = " + v + ";");
+    }
+    q[r] = s[r] = false;
+  }
+  void flush_all(Emitter &E) {
+    for (int r = 0; r <= kAll; ++r) flush(E, r);
+  }
+  // takes the op, or flushes what it would mix and returns false: the caller emits it
+  bool take(Emitter &E, const OpDesc &op, int kind) {
+    auto entry = [&](int k) {
+      char buf[48];
+      snprintf(buf, sizeof buf, "f2(M4[%d], %d)", (op.mat + k) >> 1, (op.mat + k) & 1);
+      return std::string(buf);
+    };
+    const std::string one = "make_float2(1.f, 0.f)";
+    switch (op.type) {
+      case OP_D1: {
+        if (op.a_kind == SRC_REG) return false;
+        const std::string c = cond_expr(op.a_kind, op.a_pos);
+        if (kind == TN_GATE_Z) sign(E, kAll, c);
+        else if (kind == KIND_P || kind == TN_GATE_S || kind == TN_GATE_SDG || kind == TN_GATE_T || kind == TN_GATE_TDG)
+          phase(E, kAll, c, entry(1), one);
+        else phase(E, kAll, c, entry(1), entry(0));
+        return true;
+      }
+      case OP_CZ:
+      case OP_DP: {
+        const bool ra = op.a_kind == SRC_REG, rb = op.b_kind == SRC_REG;
+        if (ra && rb) return false;
+        std::string c;
+        if (!ra) c = cond_expr(op.a_kind, op.a_pos);
+        if (!rb) c += (c.empty() ? "" : " & ") + cond_expr(op.b_kind, op.b_pos);
+        const int r = ra ? op.a_pos : rb ? op.b_pos : kAll;
+        if (op.type == OP_CZ) sign(E, r, c);
+        else phase(E, r, c, entry(0), one);
+        return true;
+      }
+      case OP_G1: flush(E, op.a_pos); return false;
+      case OP_G2: flush(E, op.a_pos); flush(E, op.b_pos); return false;
+      default: flush(E, op.b_pos); return false;  // OP_C1: its target
+    }
+  }
+};
+
 }  // namespace
 
 // Forward pass kernels read their matrix entries from a per-pass __constant__ table when one
@@ -519,7 +603,11 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
       snprintf(buf, sizeof buf, "      a[%d] = sm[pb ^ %d];", j, ro[j]);
       E.line(buf);
     }
-    for (int o = d.op_begin; o < d.op_end; ++o) emit_op(E, p.fwd.ops[o], op_kind[o]);
+    Deferred deferred;
+    const bool defer = p.opts.target != TN_TARGET_EXPECTATION;
+    for (int o = d.op_begin; o < d.op_end; ++o)
+      if (!defer || !deferred.take(E, p.fwd.ops[o], op_kind[o])) emit_op(E, p.fwd.ops[o], op_kind[o]);
+    deferred.flush_all(E);
     for (int j = 0; j < E.R; ++j) {
       snprintf(buf, sizeof buf, "      sm[pb ^ %d] = a[%d];", ro[j], j);
       E.line(buf);
