@@ -416,9 +416,17 @@ bool jit_const_mats(const tn_plan &p) {
 
 namespace {
 
+// Forward pass kernel: one tile per CTA.  The hardware hands out tiles as CTAs finish.  (Persistent CTAs
+// with a double-buffered share of the tiles each were slower: the CTAs of an SM do not progress evenly,
+// and the last ones ran with few warps beside them; 24-qubit brickwork 1182 us, one tile per CTA 1079.)
+// The last phase stores its registers to global memory, and in passes without 4x4 blocks the first one
+// loads them from there, where a warp's lanes cover whole 32-byte sectors (tile bits 0 and 1 are thread
+// bits of the phase); otherwise the tile is staged through shared memory, as it is between phases.  (With
+// blocks the asynchronous copy is better: 24-qubit brickwork 1060 us, 1098 loaded directly; 20-qubit
+// ansatz, 64 sets, without them: 22.0 and 21.7 ms.)
 std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, int *threads_out, size_t *smem_out) {
   const PassDesc &pd = p.fwd.passes[pi];
-  const int T = pd.T, K = pd.K, L = T < kLowBits ? T : kLowBits;
+  const int T = pd.T, K = pd.K;
   const int NTHR = 1 << (T - K);
   const int TILE = 1 << T;
   const int N = p.n;
@@ -432,12 +440,13 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
   // constant cache, no shared-memory copy and no registers to hold them.  Otherwise staged in
   // shared memory per batch element.
   const bool cmem = jit_const_mats(p);
-  // resident CTAs per SM requested from the register allocator (TNQ_JIT_MIN_BLOCKS overrides): three
-  // when the entries come from constant memory (a few spilled registers, but a third CTA covers
-  // another's barriers and tile loads: 1% faster alone, 7% on the serving mix, whose wide circuits share
-  // the SMs across streams); two when each batch element's entries are staged in shared memory (the
-  // 64-set adjoint configuration's forward passes ran 8% slower at three)
-  int min_blocks = cmem ? 3 : 2;
+  // whether the pass holds precontracted 4x4 blocks, the ops that fill the registers
+  bool blocks = false;
+  for (int o = pd.op_begin; o < pd.op_end; ++o) blocks |= (p.fwd.ops[o].flags & OPF_PACKED) != 0;
+  // resident CTAs per SM requested from the register allocator (TNQ_JIT_MIN_BLOCKS overrides): four without
+  // blocks; with them three, two when their entries are staged in shared memory (18 qubits, one set: 41 us
+  // with two, 66 with three; 24 qubits from constant memory 1195, 1060 and 1122 us with two, three and four)
+  int min_blocks = !blocks ? 4 : cmem ? 3 : 2;
   if (p.is_lean) min_blocks = std::max(1, std::min(4, 1024 / NTHR));
   if (const char *mb = getenv("TNQ_JIT_MIN_BLOCKS")) min_blocks = std::max(1, std::min(4, atoi(mb)));
   if (cmem) {
@@ -453,80 +462,44 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
   // launched as programmatic dependents: wait for the previous pass before any memory access
   E.line("  asm volatile(\"griddepcontrol.wait;\" ::: \"memory\");");
   E.line("  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");");
-  const int nbuf = pd.init_mode ? 1 : 2;  // loaded passes double-buffer their tiles
-  E.line("  float2 *const sm0 = reinterpret_cast<float2 *>(smraw);");
-  snprintf(buf, sizeof buf, "  float2 *const sm1 = sm0 + %d;", (nbuf - 1) * TILE);
-  E.line(buf);
+  E.line("  float2 *const sm = reinterpret_cast<float2 *>(smraw);");
   if (!cmem) {
-    snprintf(buf, sizeof buf, "  float4 *smat = reinterpret_cast<float4 *>(sm0 + %d);", nbuf * TILE);
+    snprintf(buf, sizeof buf, "  float4 *smat = reinterpret_cast<float4 *>(sm + %d);", TILE);
     E.line(buf);
   }
   E.line("  const int tid = threadIdx.x;");
-  // per-thread part of the load/store deposit: tile index i = 2*tid + 2*k*NTHR
-  {
+  const int chunks = TILE / 2 / NTHR;
+  // state offset of tile index 2 tid + 2 k NTHR (the coalesced copies) and its shared-memory position
+  auto emit_copy_base = [&]() {
     std::string dep = "0ll";
     for (int j = 1; j <= T - K; ++j) {
       snprintf(buf, sizeof buf, " | ((long long)((tid >> %d) & 1) << %d)", j - 1, (int)pd.tile_pos[j]);
       dep += buf;
     }
-    E.line("  const long long dep_t = " + dep + ";");
-    E.line("  const int sw_t = swz(2 * tid);");
-  }
-  E.line("  long long cur_b = -1;");
-  const int chunks = TILE / 2 / NTHR;
-  auto emit_base = [&](const char *tv, const char *bv) {
-    std::string base = "0ull";
-    for (int j = 0; j < pd.n_outer; ++j) {
-      snprintf(buf, sizeof buf, " | ((u64)((%s >> %d) & 1) << %d)", tv, j, (int)pd.outer_pos[j]);
-      base += buf;
-    }
-    return std::string("const u64 ") + bv + " = " + base + ";";
+    E.line("      const long long dep_t = " + dep + ";");
+    E.line("      const int sw_t = swz(2 * tid);");
   };
-  if (!pd.init_mode) {
-    // asynchronous copy of one tile into a buffer (8-byte cp.async keeps the element swizzle)
-    E.line("  auto issue = [&](long long w2, float2 *dst) {");
-    snprintf(buf, sizeof buf, "    const long long b2 = w2 >> %d; const long long t2 = w2 & %lldll;", pd.n_outer,
-             (long long)((1ll << pd.n_outer) - 1));
-    E.line(buf);
-    E.line("    " + emit_base("t2", "base2"));
-    snprintf(buf, sizeof buf, "    const float2 *src = state + (b2 << %d) + base2 + dep_t;", N);
-    E.line(buf);
-    E.line("    const unsigned d0 = (unsigned)__cvta_generic_to_shared(dst);");
-    for (int k = 0; k < chunks; ++k) {
-      const int ik = 2 * k * NTHR;
-      long long depk = 0;
-      for (int j = 0; j < T; ++j)
-        if ((ik >> j) & 1) depk |= 1ll << pd.tile_pos[j];
-      const int swk = swz_host(ik);
-      snprintf(buf, sizeof buf,
-               "    asm volatile(\"cp.async.ca.shared.global [%%0], [%%1], 8;\" :: \"r\"(d0 + 8u * (unsigned)(sw_t ^ %d)), \"l\"(src + %lldll));",
-               swk, depk);
-      E.line(buf);
-      snprintf(buf, sizeof buf,
-               "    asm volatile(\"cp.async.ca.shared.global [%%0], [%%1], 8;\" :: \"r\"(d0 + 8u * (unsigned)(sw_t ^ %d ^ 1)), \"l\"(src + %lldll + 1));",
-               swk, depk);
-      E.line(buf);
-    }
-    E.line("  };");
-    E.line("  if (blockIdx.x < work) issue(blockIdx.x, sm0);");
-    E.line("  asm volatile(\"cp.async.commit_group;\" ::: \"memory\");");
-  }
-  E.line("  int cur = 0;");
-  snprintf(buf, sizeof buf, "  for (long long w = blockIdx.x; w < work; w += gridDim.x) {");
-  E.line(buf);
-  E.line("    float2 *const sm = cur ? sm1 : sm0;");
+  auto copy_off = [&](int k) {
+    const int ik = 2 * k * NTHR;
+    long long depk = 0;
+    for (int j = 0; j < T; ++j)
+      if ((ik >> j) & 1) depk |= 1ll << pd.tile_pos[j];
+    return depk;
+  };
+  E.line("  long long cur_b = -1;");
+  E.line("  for (long long w = blockIdx.x; w < work; w += gridDim.x) {");
   snprintf(buf, sizeof buf, "    const long long b = w >> %d; const long long t = w & %lldll;", pd.n_outer,
            (long long)((1ll << pd.n_outer) - 1));
   E.line(buf);
-  E.line("    " + emit_base("t", "base"));
-  if (!pd.init_mode) {
-    // prefetch the next tile into the other buffer, then wait for this one
-    E.line("    if (w + gridDim.x < work) issue(w + gridDim.x, cur ? sm0 : sm1);");
-    E.line("    asm volatile(\"cp.async.commit_group;\" ::: \"memory\");");
-    E.line("    asm volatile(\"cp.async.wait_group 1;\" ::: \"memory\");");
-    E.line("    __syncthreads();");
+  {
+    std::string base = "0ull";
+    for (int j = 0; j < pd.n_outer; ++j) {
+      snprintf(buf, sizeof buf, " | ((u64)((t >> %d) & 1) << %d)", j, (int)pd.outer_pos[j]);
+      base += buf;
+    }
+    E.line("    const u64 base = " + base + ";");
   }
-  snprintf(buf, sizeof buf, "    float2 *st = state + (b << %d);", N);
+  snprintf(buf, sizeof buf, "    float2 *const st = state + (b << %d) + base;", N);
   E.line(buf);
   if (pd.init_mode && pd.n_outer > 0) {
     // a basis state is zero outside the one tile that holds it: store zeros, skip the phases
@@ -534,13 +507,10 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
     for (int j = 0; j < pd.n_outer; ++j) outer_mask |= 1ull << pd.outer_pos[j];
     snprintf(buf, sizeof buf, "    if ((init_basis & %lluull) != base) {", outer_mask);
     E.line(buf);
+    emit_copy_base();
     for (int k = 0; k < chunks; ++k) {
-      const int ik = 2 * k * NTHR;
-      long long depk = 0;
-      for (int j = 0; j < T; ++j)
-        if ((ik >> j) & 1) depk |= 1ll << pd.tile_pos[j];
-      snprintf(buf, sizeof buf,
-               "      *reinterpret_cast<float4 *>(st + base + dep_t + %lldll) = make_float4(0.f, 0.f, 0.f, 0.f);", depk);
+      snprintf(buf, sizeof buf, "      *reinterpret_cast<float4 *>(st + dep_t + %lldll) = make_float4(0.f, 0.f, 0.f, 0.f);",
+               copy_off(k));
       E.line(buf);
     }
     E.line("      continue;");
@@ -558,49 +528,79 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
     snprintf(buf, sizeof buf, "      for (int i = tid; i < %d; i += %d) smat[i] = src[i];", mat_n / 2, NTHR);
     E.line(buf);
     E.line("      cur_b = b;");
-    E.line("      __syncthreads();");
     E.line("    }");
     snprintf(buf, sizeof buf, "    const float4 *M4 = smat - %d;", pd.mat_begin / 2);
     E.line(buf);
   }
-  // synthesise the first pass's tile (loaded passes were filled by cp.async above)
-  if (pd.init_mode) {
-    snprintf(buf, sizeof buf, "    for (int i = tid; i < %d; i += %d) sm[i] = make_float2(0.f, 0.f);", TILE, NTHR);
-    E.line(buf);
-    E.line("    __syncthreads();");
-    unsigned long long outer_mask = 0;
-    for (int j = 0; j < pd.n_outer; ++j) outer_mask |= 1ull << pd.outer_pos[j];
-    snprintf(buf, sizeof buf, "    if (tid == 0 && (init_basis & %lluull) == base) {", outer_mask);
-    E.line(buf);
-    std::string li = "0";
-    for (int j = 0; j < T; ++j) {
-      snprintf(buf, sizeof buf, " | ((int)((init_basis >> %d) & 1ull) << %d)", (int)pd.tile_pos[j], j);
-      li += buf;
-    }
-    E.line("      const int li = " + li + ";");
-    E.line("      sm[swz(li)] = make_float2(1.f, 0.f);");
-    E.line("    }");
-    E.line("    __syncthreads();");
+  // a pass without gates (the first of an empty circuit) still writes its tile: one phase without ops
+  std::vector<PhaseDesc> phases(p.fwd.phases.begin() + pd.phase_begin, p.fwd.phases.begin() + pd.phase_end);
+  if (phases.empty()) {
+    PhaseDesc d;
+    std::memset(&d, 0, sizeof(d));
+    for (int r = 0; r < K; ++r) d.reg_pos[r] = (uint8_t)(T - K + r);
+    for (int j = 0; j < T - K; ++j) d.thr_pos[j] = (uint8_t)j;
+    phases.push_back(d);
   }
-  // phases
-  for (int ph = pd.phase_begin; ph < pd.phase_end; ++ph) {
-    const PhaseDesc &d = p.fwd.phases[ph];
+  auto direct = [&](const PhaseDesc &d) {
+    for (int r = 0; r < K; ++r)
+      if (d.reg_pos[r] < 2) return false;
+    return true;
+  };
+  const bool load_staged = !pd.init_mode && (blocks || !direct(phases.front())), store_staged = !direct(phases.back());
+  if (load_staged) {
+    // asynchronous copy of the tile (8 bytes each keeps the element swizzle)
     E.line("    {");
-    std::string tb = "0";
+    emit_copy_base();
+    E.line("      const unsigned d0 = (unsigned)__cvta_generic_to_shared(sm);");
+    E.line("      const float2 *const src = st + dep_t;");
+    for (int k = 0; k < chunks; ++k)
+      for (int h = 0; h < 2; ++h) {
+        snprintf(buf, sizeof buf,
+                 "      asm volatile(\"cp.async.ca.shared.global [%%0], [%%1], 8;\" :: \"r\"(d0 + 8u * (unsigned)(sw_t ^ %d)), \"l\"(src + %lldll));",
+                 swz_host(2 * k * NTHR) ^ h, copy_off(k) + h);
+        E.line(buf);
+      }
+    E.line("      asm volatile(\"cp.async.commit_group;\" ::: \"memory\");");
+    E.line("      asm volatile(\"cp.async.wait_group 0;\" ::: \"memory\");");
+    E.line("    }");
+  }
+  if (load_staged || !cmem) E.line("    __syncthreads();");
+  for (size_t ph = 0; ph < phases.size(); ++ph) {
+    const PhaseDesc &d = phases[ph];
+    const bool first = ph == 0, last = ph + 1 == phases.size();
+    E.line("    {");
+    std::string tb = "0", gb = "0ll";
     for (int j = 0; j < T - K; ++j) {
       snprintf(buf, sizeof buf, " | (((tid >> %d) & 1) << %d)", j, (int)d.thr_pos[j]);
       tb += buf;
+      snprintf(buf, sizeof buf, " | ((long long)((tid >> %d) & 1) << %d)", j, (int)pd.tile_pos[d.thr_pos[j]]);
+      gb += buf;
     }
     E.line("      const int tb = " + tb + ";");
     E.line("      const int pb = swz(tb);");
+    const bool from_global = first && !pd.init_mode && !load_staged, to_global = last && !store_staged;
+    if (from_global || to_global) E.line("      float2 *const gt = st + (" + gb + ");");
+    if (first && pd.init_mode) {
+      std::string li = "0";
+      for (int j = 0; j < T; ++j) {
+        snprintf(buf, sizeof buf, " | ((int)((init_basis >> %d) & 1ull) << %d)", (int)pd.tile_pos[j], j);
+        li += buf;
+      }
+      E.line("      const int li = (" + li + ") ^ tb;");  // the tile is the one that holds the basis state
+    }
     E.line("      float2 a[" + std::to_string(E.R) + "];");
-    int ro[32];
+    std::vector<int> ro(E.R), off(E.R, 0);
+    std::vector<long long> go(E.R, 0);
     for (int j = 0; j < E.R; ++j) {
-      int off = 0;
       for (int r = 0; r < K; ++r)
-        if ((j >> r) & 1) off |= 1 << d.reg_pos[r];
-      ro[j] = swz_host(off);
-      snprintf(buf, sizeof buf, "      a[%d] = sm[pb ^ %d];", j, ro[j]);
+        if ((j >> r) & 1) {
+          off[j] |= 1 << d.reg_pos[r];
+          go[j] |= 1ll << pd.tile_pos[d.reg_pos[r]];
+        }
+      ro[j] = swz_host(off[j]);
+      if (first && pd.init_mode) snprintf(buf, sizeof buf, "      a[%d] = make_float2(li == %d ? 1.f : 0.f, 0.f);", j, off[j]);
+      else if (from_global) snprintf(buf, sizeof buf, "      a[%d] = gt[%lldll];", j, go[j]);
+      else snprintf(buf, sizeof buf, "      a[%d] = sm[pb ^ %d];", j, ro[j]);
       E.line(buf);
     }
     Deferred deferred;
@@ -609,32 +609,31 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
       if (!defer || !deferred.take(E, p.fwd.ops[o], op_kind[o])) emit_op(E, p.fwd.ops[o], op_kind[o]);
     deferred.flush_all(E);
     for (int j = 0; j < E.R; ++j) {
-      snprintf(buf, sizeof buf, "      sm[pb ^ %d] = a[%d];", ro[j], j);
+      if (to_global) snprintf(buf, sizeof buf, "      gt[%lldll] = a[%d];", go[j], j);
+      else snprintf(buf, sizeof buf, "      sm[pb ^ %d] = a[%d];", ro[j], j);
       E.line(buf);
     }
     E.line("    }");
     E.line("    __syncthreads();");
   }
-  // store
-  for (int k = 0; k < chunks; ++k) {
-    const int ik = 2 * k * NTHR;
-    long long depk = 0;
-    for (int j = 0; j < T; ++j)
-      if ((ik >> j) & 1) depk |= 1ll << pd.tile_pos[j];
-    const int swk = swz_host(ik);
-    snprintf(buf, sizeof buf,
-             "    { const float2 x = sm[sw_t ^ %d], y = sm[sw_t ^ %d ^ 1]; "
-             "*reinterpret_cast<float4 *>(st + base + dep_t + %lldll) = make_float4(x.x, x.y, y.x, y.y); }",
-             swk, swk, depk);
-    E.line(buf);
+  if (store_staged) {
+    E.line("    {");
+    emit_copy_base();
+    for (int k = 0; k < chunks; ++k) {
+      const int swk = swz_host(2 * k * NTHR);
+      snprintf(buf, sizeof buf,
+               "      { const float2 x = sm[sw_t ^ %d], y = sm[sw_t ^ %d ^ 1]; "
+               "*reinterpret_cast<float4 *>(st + dep_t + %lldll) = make_float4(x.x, x.y, y.x, y.y); }",
+               swk, swk, copy_off(k));
+      E.line(buf);
+    }
+    E.line("    }");
+    E.line("    __syncthreads();");
   }
-  E.line("    __syncthreads();");
-  E.line("    cur ^= 1;");
   E.line("  }");
-  if (!pd.init_mode) E.line("  asm volatile(\"cp.async.wait_group 0;\" ::: \"memory\");");
   E.line("}");
   *threads_out = NTHR;
-  *smem_out = (size_t)nbuf * TILE * 8 + (cmem ? 0 : (size_t)mat_n * 8);
+  *smem_out = (size_t)TILE * 8 + (cmem ? 0 : (size_t)mat_n * 8);
   return E.o.str();
 }
 

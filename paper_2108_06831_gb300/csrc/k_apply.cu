@@ -9,6 +9,8 @@
 // maps K tile bits to registers and applies its ops there) and writes the tile back.
 // Tiles are independent, so the grid is persistent: one wave of CTAs sized from the
 // occupancy calculator, striding over batch x 2^(N-T) tiles.
+#include <algorithm>
+
 #include "apply_common.cuh"
 #include "kernels.h"
 
@@ -173,11 +175,9 @@ cudaError_t launch_forward(const tn_plan *p, const float2 *mats, long long mstri
       const PassDesc &h = p->fwd.passes[i];
       const int threads = p->jit_threads[i];
       const size_t smem = p->jit_smem[i];
-      const int per_sm = i < p->jit_grid.size() ? p->jit_grid[i] : 1;  // resident CTAs per SM (load time)
       cudaError_t e = cudaSuccess;
       long long work = (long long)p->batch << h.n_outer;
-      long long grid = (long long)num_sms() * per_sm;
-      if (grid > work) grid = work;
+      const long long grid = std::min<long long>(work, 1ll << 30);  // one tile per CTA
       const float2 *m = mats;
       unsigned long long init = p->init;
       // per-call tables (parameterised, batch 1): this pass's entries into its constant table
