@@ -903,6 +903,14 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
     depk[k] = d;
     swk[k] = swz_host(ik);
   }
+  // the first phase loads and the last one stores its registers directly where a warp's lanes cover whole
+  // 32-byte sectors (as in the forward passes)
+  auto direct = [&](const PhaseDesc &d) {
+    for (int r = 0; r < K; ++r)
+      if (d.reg_pos[r] < 2) return false;
+    return true;
+  };
+  const bool load_staged = !direct(p.bwd.phases[pd.phase_begin]), store_staged = !direct(p.bwd.phases[pd.phase_end - 1]);
   E.line("  auto issue = [&](long long t2, float2 *dp, float2 *dl) {");
   E.line("    " + emit_base("t2", "base2"));
   E.line("    const float2 *sp = gp + base2 + dep_t; const float2 *sl = gl + base2 + dep_t;");
@@ -925,9 +933,11 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
   E.line(buf);
   E.line("    float2 *const smp = p0; float2 *const sml = l0;");
   E.line("    " + emit_base("t", "base"));
-  E.line("    issue(t, p0, l0);");
-  E.line("    asm volatile(\"cp.async.commit_group;\" ::: \"memory\");");
-  E.line("    asm volatile(\"cp.async.wait_group 0;\" ::: \"memory\");");
+  if (load_staged) {
+    E.line("    issue(t, p0, l0);");
+    E.line("    asm volatile(\"cp.async.commit_group;\" ::: \"memory\");");
+    E.line("    asm volatile(\"cp.async.wait_group 0;\" ::: \"memory\");");
+  }
   E.line("    __syncthreads();");
   // the next tile on its way to L2 while this one is computed
   E.line("    if (t + gridDim.x < " + std::to_string(NT) + "ll) {");
@@ -956,14 +966,29 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
     }
     E.line("      const int tb = " + tb + ";");
     E.line("      const int pb = swz(tb);");
+    const bool from_global = ph == pd.phase_begin && !load_staged, to_global = ph + 1 == pd.phase_end && !store_staged;
+    if (from_global || to_global) {
+      std::string gb = "0ll";
+      for (int j = 0; j < T - K; ++j) {
+        snprintf(buf, sizeof buf, " | ((long long)((tid >> %d) & 1) << %d)", j, (int)pd.tile_pos[d.thr_pos[j]]);
+        gb += buf;
+      }
+      E.line("      const long long gt = (long long)base + (" + gb + ");");
+    }
     E.line("      float2 a[" + std::to_string(E.R) + "], l[" + std::to_string(E.R) + "];");
     int ro[32];
+    long long go[32];
     for (int j = 0; j < E.R; ++j) {
       int off = 0;
+      go[j] = 0;
       for (int r = 0; r < K; ++r)
-        if ((j >> r) & 1) off |= 1 << d.reg_pos[r];
+        if ((j >> r) & 1) {
+          off |= 1 << d.reg_pos[r];
+          go[j] |= 1ll << pd.tile_pos[d.reg_pos[r]];
+        }
       ro[j] = swz_host(off);
-      snprintf(buf, sizeof buf, "      a[%d] = smp[pb ^ %d]; l[%d] = sml[pb ^ %d];", j, ro[j], j, ro[j]);
+      if (from_global) snprintf(buf, sizeof buf, "      a[%d] = gp[gt + %lldll]; l[%d] = gl[gt + %lldll];", j, go[j], j, go[j]);
+      else snprintf(buf, sizeof buf, "      a[%d] = smp[pb ^ %d]; l[%d] = sml[pb ^ %d];", j, ro[j], j, ro[j]);
       E.line(buf);
     }
     std::vector<PendingDot> dots;
@@ -992,13 +1017,14 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
     }
     emit_dot_sums(E, dots, NW);
     for (int j = 0; j < E.R; ++j) {
-      snprintf(buf, sizeof buf, "      smp[pb ^ %d] = a[%d]; sml[pb ^ %d] = l[%d];", ro[j], j, ro[j], j);
+      if (to_global) snprintf(buf, sizeof buf, "      gp[gt + %lldll] = a[%d]; gl[gt + %lldll] = l[%d];", go[j], j, go[j], j);
+      else snprintf(buf, sizeof buf, "      smp[pb ^ %d] = a[%d]; sml[pb ^ %d] = l[%d];", ro[j], j, ro[j], j);
       E.line(buf);
     }
     E.line("    }");
     E.line("    __syncthreads();");
   }
-  for (int k = 0; k < chunks; ++k) {
+  for (int k = 0; k < chunks && store_staged; ++k) {
     snprintf(buf, sizeof buf,
              "    { const float2 x = smp[sw_t ^ %d], y = smp[sw_t ^ %d ^ 1]; "
              "*reinterpret_cast<float4 *>(gp + base + dep_t + %lldll) = make_float4(x.x, x.y, y.x, y.y); "

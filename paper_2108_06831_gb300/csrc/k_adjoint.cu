@@ -8,6 +8,8 @@
 // conjugate-transposed tables, grouped into passes and register phases the same way,
 // with two tiles (psi, lambda) staged per CTA.  Derivative dots are reduced in FP32 per
 // warp, accumulated per CTA in FP64 in shared memory, and added to grad once per CTA.
+#include <algorithm>
+
 #include "apply_common.cuh"
 #include "kernels.h"
 
@@ -238,7 +240,9 @@ cudaError_t launch_backward(const tn_plan *p, const float2 *mats, long long mstr
       const int per_sm = i < p->jit_bwd_grid.size() ? p->jit_bwd_grid[i] : 1;  // queried at load time
       cudaError_t e = cudaSuccess;
       const long long n_tiles = 1ll << h.n_outer;
-      const long long gx = grid_per_row(n_tiles, p->batch, per_sm);
+      // about four tiles per CTA where that is many waves (2 and 4 tiles 20.7 and 20.8 ms on 20 qubits, 64
+      // sets, 16 tiles 21.9, 57 tiles in one wave 23.6: the CTAs of an SM progress unevenly)
+      const long long gx = std::max(grid_per_row(n_tiles, p->batch, per_sm), n_tiles / 4);
       const float2 *m = mats;
       int np = p->n_params;
       void *args[] = {(void *)&m, (void *)&mstride, (void *)&psi, (void *)&lam, (void *)&grad, (void *)&np};
