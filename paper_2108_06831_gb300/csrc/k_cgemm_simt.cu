@@ -5,12 +5,8 @@
 // (both operands stored with the contracted index contiguous).  This kernel is the FP32
 // reference the tensor-core forms are measured against, and the form used for merges too
 // narrow for the tensor-core tiles.  One template covers the shapes a network contraction
-// produces: a CTA of 256 threads computes a BM x BN tile in TM x TN complex blocks per
-// thread, streaming BK-deep slices of both operands through shared memory (two slices in
-// flight, copied asynchronously; rows padded so a warp's reads fall in distinct banks), with
-// FFMA accumulation.
-// The tile is fitted to the operand shape: narrow N (down to 8 columns) takes tall tiles so
-// that no column work is wasted, and short K (8) takes an 8-deep slice.
+// produces: a CTA of 128 threads computes a BM x BN tile in TM x TN complex blocks per thread,
+// streaming 16-deep slices of K of both operands through shared memory, with FFMA accumulation.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -21,14 +17,14 @@ namespace tnq {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;  // of a tile's CTA
 
 // An output map with the tables of its permuted epilogue for one tile shape.
 struct StagedMap {
   OutMap map;
   int lgn, L, nlo, pairs;
-  int s_lo[64], s_hi[128];       // staging offsets (complex)
-  long long g_lo[64], g_hi[128];  // stored offsets (complex)
+  int s_lo[64], s_hi[64];        // staging offsets (complex)
+  long long g_lo[64], g_hi[64];  // stored offsets (complex)
 };
 void build_staged(StagedMap &sm, const OutMap &om, long long M, long long N, int BM, int BN);
 
@@ -40,10 +36,6 @@ __device__ __forceinline__ long long map_bits(const OutMap &om, long long f, int
   return r;
 }
 
-__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -54,8 +46,8 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int THREADS>
 __device__ __forceinline__ void store_staged(const float2 *smem, float2 *__restrict__ C, long long gbase,
                                              const StagedMap &om) {
-  __shared__ int s_lo[64], s_hi[128];
-  __shared__ long long g_lo[64], g_hi[128];
+  __shared__ int s_lo[64], s_hi[64];
+  __shared__ long long g_lo[64], g_hi[64];
   const int L = om.L, nlo = om.nlo, lo_mask = (1 << om.nlo) - 1;
   if (threadIdx.x < 64) {
     s_lo[threadIdx.x] = om.s_lo[threadIdx.x];
@@ -81,119 +73,22 @@ __device__ __forceinline__ void store_staged(const float2 *smem, float2 *__restr
   }
 }
 
-template <int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__(kThreads, 2) k_cgemm_fp32(long long M, long long N, long long K, long long k_len,
-                                                         const float2 *__restrict__ A, const float2 *__restrict__ B,
-                                                         float2 *__restrict__ C, float2 *__restrict__ P,
-                                                         const __grid_constant__ StagedMap om) {
-  static_assert((BM / TM) * (BN / TN) == kThreads, "one thread per TM x TN block");
-  pdl_wait();
-  pdl_trigger();
-  // two K slices of both operands in flight (row-major, row stride BK + 1: a warp's reads across
-  // rows fall in distinct banks); the C tile (row stride BN + 1) in the permuted epilogue
-  constexpr int kLd = BK + 1;
-  constexpr int kSlice = (BM + BN) * kLd, kTile = BM * (BN + 1);
-  __shared__ float2 smem[2 * kSlice > kTile ? 2 * kSlice : kTile];
-  // tiles of one batch element along x, n fastest (M may need more than 65535 row tiles)
-  const long long tiles_n = (N + BN - 1) / BN;
-  const long long b = blockIdx.z;
-  const long long m0 = ((long long)blockIdx.x / tiles_n) * BM, n0 = ((long long)blockIdx.x % tiles_n) * BN;
-  const float2 *Ab = A + b * M * K;
-  const float2 *Bb = B + b * N * K;
-  float2 *Cb = C + b * M * N;
-  // split K (P != nullptr): this CTA sums k in [kb, ke) and stores its partial tile to P
-  const long long kb = (long long)blockIdx.y * k_len, ke = kb + k_len < K ? kb + k_len : K;
-  constexpr int NX = BN / TN;  // threads along n
-  const int tx = threadIdx.x % NX, ty = threadIdx.x / NX;
-  float2 acc[TM][TN];
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  // slice k0 of A (BM rows) and B (BN rows) into buffer sb: asynchronous copies of the
-  // elements in range, zeros for the ragged edges
-  auto load_slice = [&](int sb, long long k0) {
-    float2 *as = smem + sb * kSlice, *bs = as + BM * kLd;
-    for (int e = threadIdx.x; e < (BM + BN) * BK; e += kThreads) {
-      const int r = e / BK, c = e % BK;
-      const long long gk = k0 + c;
-      if (r < BM) {
-        const long long gm = m0 + r;
-        if (gm < M && gk < ke) cp_async8(as + r * kLd + c, Ab + gm * K + gk);
-        else as[r * kLd + c] = make_float2(0.f, 0.f);
-      } else {
-        const long long gn = n0 + (r - BM);
-        if (gn < N && gk < ke) cp_async8(bs + (r - BM) * kLd + c, Bb + gn * K + gk);
-        else bs[(r - BM) * kLd + c] = make_float2(0.f, 0.f);
-      }
-    }
-    cp_async_commit();
-  };
-  int sb = 0;
-  if (ke > kb) load_slice(0, kb);
-  for (long long k0 = kb; k0 < ke; k0 += BK) {
-    if (k0 + BK < ke) {
-      load_slice(sb ^ 1, k0 + BK);
-      cp_async_wait<1>();  // the current slice has landed (the next may still be in flight)
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const float2 *as = smem + sb * kSlice, *bs = as + BM * kLd;
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float2 a[TM], bb[TN];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = as[(ty + (BM / TM) * i) * kLd + kk];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) bb[j] = bs[(tx + NX * j) * kLd + kk];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-          acc[i][j].x = fmaf(a[i].x, bb[j].x, acc[i][j].x);
-          acc[i][j].x = fmaf(-a[i].y, bb[j].y, acc[i][j].x);
-          acc[i][j].y = fmaf(a[i].x, bb[j].y, acc[i][j].y);
-          acc[i][j].y = fmaf(a[i].y, bb[j].x, acc[i][j].y);
-        }
-    }
-    __syncthreads();  // the buffer is free for the slice after next
-    sb ^= 1;
-  }
-  if (P != nullptr || om.map.identity) {
-    float2 *Ob = P != nullptr ? P + ((long long)blockIdx.y * gridDim.z + b) * M * N : Cb;
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        const long long gm = m0 + ty + (BM / TM) * i, gn = n0 + tx + NX * j;
-        if (gm < M && gn < N) Ob[gm * N + gn] = acc[i][j];
-      }
-  } else {
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TN; ++j) smem[(ty + (BM / TM) * i) * (BN + 1) + tx + NX * j] = acc[i][j];
-    store_staged<kThreads>(smem, C, map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0), om);
-  }
-}
-
-// The wide form, for outputs of more than 32 columns with enough tiles to fill the SMs: 128 x 64 tiles,
-// 128 threads of 8 x 8 complex accumulators.  What bounds the 64 x 64 form (4 x 4 accumulators) is
-// shared memory: each step of K reads TM + TN elements per thread for TM TN complex multiply-adds, 16
-// clocks of a warp's loads per 16 clocks of its FMAs; 8 x 8 reads half as much.  Bound now: FMA issue
-// (78% of issue slots).  4096^3: 11.9 -> 9.6 ms (46 -> 57.5 TFLOP/s); batch 64, 4096 x 64 x 64: 204 ->
-// 168 us.  The packed FP32x2 multiply-adds are slower here (39.5 against 57.9 TFLOP/s at 2432 x 2048 x
-// 512): every operand of the complex product has to be duplicated or swapped into a register pair, and
-// those moves take the FMA pipe's slots.  Same roundings in the same order as the 64 x 64 form.
-// Slices of 16 K are staged by cp.async, three in flight, in rows of 18 elements (16-byte aligned, a
-// warp's reads conflict-free); VEC: 16-byte copies, for even K.  Four steps of K are unrolled (2, 8 and
-// 16 measured 9.8, 9.8 and 10.3 ms).
-constexpr int kWideThreads = 128, kWideK = 16, kWideStages = 3;
-constexpr int kWideLd = kWideK + 2;
+// Tiles: the columns fitted to N (8, 16, 32 or 64), the rows by short_tiles.  Bound: FMA issue, and for
+// narrow N the loads of A beside it.  Before, 256 threads of 2 x 2 to 4 x 4 accumulators copied the slices
+// 8 bytes at a time: the copies' address arithmetic and one shared-memory load for every four multiply-adds
+// took more issue slots than the multiply-adds.  128 threads, 16-byte copies and 4 x 2 to 8 x 4 accumulators,
+// four CTAs per SM or more: batch 64, 32768 x 8 x 64: 333 -> 253 us; x 16: 488 -> 364; x 32: 894 -> 612;
+// 4096 x 64 x 64: 204 -> 156; 4096^3 11.9 -> 9.2 ms (59.6 TFLOP/s).  Slower at 4096^3: 128 x 64 tiles of
+// 8 x 8 (9.6 ms; two CTAs per SM leave a worse last wave too: 2048^3 1394 against 1217 us), two steps of K
+// per shared-memory load (9.3, spills), three slices in flight (9.8), and packed FP32x2 multiply-adds, with
+// the operands duplicated in registers (39.5 against 57.9 TFLOP/s at 2432 x 2048 x 512) or laid out in pairs
+// in shared memory (11.2 ms).
+// Slices of 16 K are staged by cp.async, two in flight, in rows of 18 elements (16-byte aligned, a
+// warp's reads conflict-free); VEC: 16-byte copies, for even K.  Four steps of K are unrolled.
+constexpr int kSliceK = 16, kLd = kSliceK + 2, kStages = 2;
 template <int BM, int BN>
-constexpr size_t wide_smem() {
-  constexpr int slices = kWideStages * (BM + BN) * kWideLd, tile = BM * (BN + 1);
+constexpr size_t tile_smem() {
+  constexpr int slices = kStages * (BM + BN) * kLd, tile = BM * (BN + 1);
   return sizeof(float2) * (slices > tile ? slices : tile);
 }
 
@@ -205,40 +100,41 @@ __device__ __forceinline__ void cp_async_z(void *dst, const void *src, int n) {
                : "memory");
 }
 
-template <bool VEC, int BM, int BN, int TM, int TN, int MINB>
-__global__ void __launch_bounds__(kWideThreads, MINB) k_cgemm_fp32_wide(long long M, long long N, long long K,
-                                                                     const float2 *__restrict__ A,
-                                                                     const float2 *__restrict__ B,
-                                                                     float2 *__restrict__ C,
-                                                                     const __grid_constant__ StagedMap om) {
-  static_assert((BM / TM) * (BN / TN) == kWideThreads, "one thread per TM x TN block");
-  constexpr int NX = BN / TN, NY = BM / TM, kSlice = (BM + BN) * kWideLd;
-  extern __shared__ __align__(16) float2 smem_w[];
+template <bool VEC, bool SPLIT, int BM, int BN, int TM, int TN, int MINB>
+__global__ void __launch_bounds__(kThreads, MINB) k_cgemm_fp32(long long M, long long N, long long K, long long k_len,
+                                                            const float2 *__restrict__ A, const float2 *__restrict__ B,
+                                                            float2 *__restrict__ C, float2 *__restrict__ P,
+                                                            const __grid_constant__ StagedMap om) {
+  static_assert((BM / TM) * (BN / TN) == kThreads, "one thread per TM x TN block");
+  static_assert(BM * BN <= 1 << 12, "StagedMap covers a tile");
+  constexpr int NX = BN / TN, NY = BM / TM, kSlice = (BM + BN) * kLd;
+  extern __shared__ __align__(16) float2 smem[];
   pdl_wait();
   pdl_trigger();
+  // tiles of one batch element along x, n fastest (M may need more than 65535 row tiles)
   const long long tiles_n = (N + BN - 1) / BN;
   const long long b = blockIdx.z;
   const long long m0 = ((long long)blockIdx.x / tiles_n) * BM, n0 = ((long long)blockIdx.x % tiles_n) * BN;
+  // SPLIT: this CTA sums k in [kb, ke) and stores its partial tile to P
+  const long long kb = SPLIT ? (long long)blockIdx.y * k_len : 0, ke = SPLIT && kb + k_len < K ? kb + k_len : K;
   const float2 *Ab = A + (b * M + m0) * K, *Bb = B + (b * N + n0) * K;
-  constexpr int kPer = VEC ? 2 : 1;                       // elements per copy
-  constexpr int kCols = kWideK / kPer;                    // copies per row
-  constexpr int kStep = kWideThreads / kCols;             // rows copied at once
+  constexpr int kPer = VEC ? 2 : 1;        // elements per copy
+  constexpr int kCols = kSliceK / kPer;    // copies per row
+  constexpr int kStep = kThreads / kCols;  // rows copied at once
   const int lr = threadIdx.x / kCols, lc = (threadIdx.x % kCols) * kPer;
   const int rows_a = (int)(M - m0 < BM ? M - m0 : BM), rows_b = (int)(N - n0 < BN ? N - n0 : BN);
+  // `most` rows of a slice of one operand: elements in range, zeros for the ragged edges
+  auto load_rows = [&](float2 *dst, const float2 *src, const float2 *base, int rows, int most, bool in_k) {
+#pragma unroll
+    for (int r = lr; r < most; r += kStep) {
+      const bool ok = in_k && r < rows;
+      cp_async_z<8 * kPer>(dst + r * kLd + lc, ok ? src + r * K : base, ok ? 8 * kPer : 0);
+    }
+  };
   auto load_slice = [&](int sb, long long k0) {
-    float2 *as = smem_w + sb * kSlice, *bs = as + BM * kWideLd;
-    const bool in_k = k0 + lc < K;
-    const float2 *ga = Ab + k0 + lc, *gb = Bb + k0 + lc;
-#pragma unroll
-    for (int r = lr; r < BM; r += kStep) {
-      const bool ok = in_k && r < rows_a;
-      cp_async_z<8 * kPer>(as + r * kWideLd + lc, ok ? ga + r * K : A, ok ? 8 * kPer : 0);
-    }
-#pragma unroll
-    for (int r = lr; r < BN; r += kStep) {
-      const bool ok = in_k && r < rows_b;
-      cp_async_z<8 * kPer>(bs + r * kWideLd + lc, ok ? gb + r * K : B, ok ? 8 * kPer : 0);
-    }
+    float2 *as = smem + sb * kSlice;
+    load_rows(as, Ab + k0 + lc, A, rows_a, BM, k0 + lc < ke);
+    load_rows(as + BM * kLd, Bb + k0 + lc, B, rows_b, BN, k0 + lc < ke);
   };
   const int tx = threadIdx.x % NX, ty = threadIdx.x / NX;
   float2 acc[TM][TN];
@@ -246,30 +142,28 @@ __global__ void __launch_bounds__(kWideThreads, MINB) k_cgemm_fp32_wide(long lon
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  const int slices = (int)((K + kWideK - 1) / kWideK);
-#pragma unroll
-  for (int t = 0; t < kWideStages - 1; ++t) {
-    if (t < slices) load_slice(t, (long long)t * kWideK);
-    cp_async_commit();
-  }
+  const int slices = (int)((ke - kb + kSliceK - 1) / kSliceK);
+  if (slices > 0) load_slice(0, kb);
+  cp_async_commit();
   for (int t = 0; t < slices; ++t) {
-    cp_async_wait<kWideStages - 2>();
+    cp_async_wait<kStages - 2>();
     __syncthreads();  // slice t has landed, and its successor's buffer (slice t - 1) is read out
-    if (t + kWideStages - 1 < slices) load_slice((t + kWideStages - 1) % kWideStages, (long long)(t + kWideStages - 1) * kWideK);
+    const long long k0 = kb + (long long)t * kSliceK;
+    if (t + 1 < slices) load_slice((t + 1) % kStages, k0 + kSliceK);
     cp_async_commit();
-    const float2 *as = smem_w + (t % kWideStages) * kSlice + ty * kWideLd;
-    const float2 *bs = smem_w + (t % kWideStages) * kSlice + (BM + tx) * kWideLd;
-    const int left = (int)(K - (long long)t * kWideK), quads = left >= kWideK ? kWideK / 4 : (left + 3) / 4;
+    const float2 *as = smem + (t % kStages) * kSlice + ty * kLd;
+    const float2 *bs = smem + (t % kStages) * kSlice + (BM + tx) * kLd;
+    const int quads = ke - k0 >= kSliceK ? kSliceK / 4 : (int)(ke - k0 + 3) / 4;
 #pragma unroll 1
     for (int q = 0; q < quads; ++q, as += 4, bs += 4)
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       float2 bb[TN];
 #pragma unroll
-      for (int j = 0; j < TN; ++j) bb[j] = bs[NX * j * kWideLd + kk];
+      for (int j = 0; j < TN; ++j) bb[j] = bs[NX * j * kLd + kk];
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
-        const float2 a = as[NY * i * kWideLd + kk];
+        const float2 a = as[NY * i * kLd + kk];
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
           acc[i][j].x = fmaf(a.x, bb[j].x, acc[i][j].x);
@@ -280,21 +174,22 @@ __global__ void __launch_bounds__(kWideThreads, MINB) k_cgemm_fp32_wide(long lon
       }
     }
   }
-  if (om.map.identity) {
+  if (SPLIT || om.map.identity) {
+    float2 *O = SPLIT ? P + ((long long)blockIdx.y * gridDim.z + b) * M * N : C + b * M * N;
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
       for (int j = 0; j < TN; ++j) {
         const long long gm = m0 + ty + NY * i, gn = n0 + tx + NX * j;
-        if (gm < M && gn < N) C[(b * M + gm) * N + gn] = acc[i][j];
+        if (gm < M && gn < N) O[gm * N + gn] = acc[i][j];
       }
   } else {
     __syncthreads();  // the last slice is read out; nothing is in flight
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < TN; ++j) smem_w[(ty + NY * i) * (BN + 1) + tx + NX * j] = acc[i][j];
-    store_staged<kWideThreads>(smem_w, C, map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0), om);
+      for (int j = 0; j < TN; ++j) smem[(ty + NY * i) * (BN + 1) + tx + NX * j] = acc[i][j];
+    store_staged<kThreads>(smem, C, map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0), om);
   }
 }
 
@@ -412,7 +307,7 @@ void build_staged(StagedMap &sm, const OutMap &om, long long M, long long N, int
   sm.pairs = L > 0 && spos(order[0]) == 0;
 }
 
-// Tile shape (BM x BN) for an output of N columns.
+// Tile shape (BM x BN) by which an output of N columns is counted: the split of K and the planner's tile fill.
 inline void tile_for(long long N, int *bm, int *bn) {
   *bn = N <= 8 ? 8 : N <= 16 ? 16 : N <= 32 ? 32 : 64;
   *bm = *bn == 64 ? 64 : 128;
@@ -438,21 +333,25 @@ int split_k(long long batch, long long M, long long N, long long K, long long *k
   return (int)((K + kl - 1) / kl);
 }
 
-template <int BM, int BN, int BK, int TM, int TN>
-cudaError_t launch_shape(long long batch, long long M, long long N, long long K, const float2 *A, const float2 *B,
+template <bool SPLIT, int BM, int BN, int TM, int TN, int MINB>
+cudaError_t launch_tiles(long long batch, long long M, long long N, long long K, const float2 *A, const float2 *B,
                          float2 *C, float2 *P, const OutMap &om, cudaStream_t s) {
   const long long tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
   if (tiles > 0x7fffffffll) return cudaErrorNotSupported;
   long long k_len = K;
-  const int splits = P != nullptr ? split_k(batch, M, N, K, &k_len) : 1;
+  const int splits = SPLIT ? split_k(batch, M, N, K, &k_len) : 1;
   dim3 grid((unsigned)tiles, (unsigned)splits, (unsigned)batch);
   StagedMap sm;
   std::memset(&sm, 0, sizeof(sm));
   sm.map = om;
-  if (!om.identity && splits == 1) build_staged(sm, om, M, N, BM, BN);
-  cudaError_t e = launch_pdl(k_cgemm_fp32<BM, BN, BK, TM, TN>, grid, dim3(kThreads), 0, s, M, N, K, k_len, A, B, C,
-                             splits > 1 ? P : (float2 *)nullptr, sm);
-  if (e != cudaSuccess || splits == 1) return e;
+  if (!om.identity && !SPLIT) build_staged(sm, om, M, N, BM, BN);
+  const bool vec = K % 2 == 0 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
+  auto *fn = vec ? k_cgemm_fp32<true, SPLIT, BM, BN, TM, TN, MINB>
+                 : k_cgemm_fp32<false, SPLIT, BM, BN, TM, TN, MINB>;
+  constexpr size_t bytes = tile_smem<BM, BN>();
+  static_assert(bytes <= 48 * 1024, "no attribute is set");
+  cudaError_t e = launch_pdl(fn, grid, dim3(kThreads), bytes, s, M, N, K, k_len, A, B, C, P, sm);
+  if (e != cudaSuccess || !SPLIT) return e;
   const long long total = batch * M * N;
   if (total <= 4096)
     return launch_pdl(k_splitk_reduce_few, dim3((unsigned)total), dim3(128), 0, s, (const float2 *)P, splits, total, C,
@@ -461,45 +360,17 @@ cudaError_t launch_shape(long long batch, long long M, long long N, long long K,
                     (const float2 *)P, splits, total, C, om);
 }
 
-// Whether the 128 x 64 form is the faster one: both it and the 64 x 64 form run two CTAs per SM, a full
-// wave of the 64 x 64 form (half the outputs) takes 0.63 of a full wave of the wide form (46 against 58
-// TFLOP/s at 4096^3), and a last wave of at most one CTA per SM about 0.6 of a full one.  Taken when that
-// estimate gains a tenth: 1500 x 1500 x 100 54.6 -> 39.5 us; below it, for instance at 40 x 200 x 200 x
-// 200, the wide form was slower (117 against 137 us).
-bool wide_ok(long long batch, long long M, long long N) {
-  const long long slots = 2ll * num_sms();
-  auto waves = [&](long long bm, long long bn) {
-    const long long tiles = batch * ((M + bm - 1) / bm) * ((N + bn - 1) / bn), r = tiles % slots;
-    return (double)(tiles / slots) + (r == 0 ? 0.0 : 2 * r <= slots ? 0.6 : 1.0);
+// Whether 32-row tiles are faster than `rows`-row ones for `tiles` column tiles (of all batch elements):
+// when the SM with the most rows has so many fewer of them that it makes up for their lower rate, `rate` of
+// the larger tiles' (32768 rows, batch 64: 0.8 at 8 to 32 columns; 4096^3: 0.96, less where tiles are short).
+// 2048 x 32 x 450: 53 and 20 us; 500^3: 58 and 38; 40 x 200 x 200 x 200: 92 and 76; the other way
+// 1000 x 1000 x 300: 60 and 77; 32 x 2048 x 32 x 32: 14.7 and 15.7.
+bool short_tiles(long long M, long long tiles, long long rows, double rate) {
+  auto most = [&](long long bm) {
+    const long long sms = num_sms();
+    return (double)((tiles * ((M + bm - 1) / bm) + sms - 1) / sms * bm);
   };
-  return M > 64 && waves(128, 64) < 0.9 * 0.63 * waves(64, 64);
-}
-template <int BM, int BN, int TM, int TN, int MINB>
-cudaError_t launch_wide(long long batch, long long M, long long N, long long K, const float2 *A, const float2 *B,
-                        float2 *C, const OutMap &om, cudaStream_t s) {
-  const long long tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  if (tiles > 0x7fffffffll || K > (1ll << 30)) return cudaErrorNotSupported;
-  StagedMap sm;
-  std::memset(&sm, 0, sizeof(sm));
-  sm.map = om;
-  if (!om.identity) build_staged(sm, om, M, N, BM, BN);
-  const bool vec = K % 2 == 0 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
-  auto *fn = vec ? k_cgemm_fp32_wide<true, BM, BN, TM, TN, MINB> : k_cgemm_fp32_wide<false, BM, BN, TM, TN, MINB>;
-  constexpr size_t smem = wide_smem<BM, BN>();
-  cudaError_t e = ensure_smem(reinterpret_cast<const void *>(fn), smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(fn, dim3((unsigned)tiles, 1, (unsigned)batch), dim3(kWideThreads), smem, s, M, N, K, A, B, C, sm);
-}
-
-template <int BK>
-cudaError_t launch_k(long long batch, long long M, long long N, long long K, const float2 *A, const float2 *B,
-                     float2 *C, float2 *P, const OutMap &om, cudaStream_t s) {
-  int bm = 0, bn = 0;
-  tile_for(N, &bm, &bn);
-  if (bn == 8) return launch_shape<128, 8, BK, 2, 2>(batch, M, N, K, A, B, C, P, om, s);
-  if (bn == 16) return launch_shape<128, 16, BK, 4, 2>(batch, M, N, K, A, B, C, P, om, s);
-  if (bn == 32) return launch_shape<128, 32, BK, 4, 4>(batch, M, N, K, A, B, C, P, om, s);
-  return launch_shape<64, 64, BK, 4, 4>(batch, M, N, K, A, B, C, P, om, s);
+  return most(32) < rate * most(rows);
 }
 
 }  // namespace
@@ -535,9 +406,24 @@ cudaError_t launch_cgemm_fp32(long long batch, long long M, long long N, long lo
     const long long blocks = std::min<long long>((total + 255) / 256, (long long)num_sms() * 16);
     return launch_pdl(k_cgemm_small, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, m);
   }
-  if (P == nullptr && N > 32 && wide_ok(batch, M, N)) return launch_wide<128, 64, 8, 8, 2>(batch, M, N, K, A, B, C, m, s);
-  if (K <= 8) return launch_k<8>(batch, M, N, K, A, B, C, P, m, s);
-  return launch_k<16>(batch, M, N, K, A, B, C, P, m, s);
+  if (P != nullptr) {  // few tiles: the short ones
+    if (N <= 8) return launch_tiles<true, 32, 8, 2, 1, 8>(batch, M, N, K, A, B, C, P, m, s);
+    if (N <= 16) return launch_tiles<true, 32, 16, 2, 2, 8>(batch, M, N, K, A, B, C, P, m, s);
+    if (N <= 32) return launch_tiles<true, 32, 32, 4, 2, 8>(batch, M, N, K, A, B, C, P, m, s);
+    return launch_tiles<true, 32, 64, 4, 4, 6>(batch, M, N, K, A, B, C, P, m, s);
+  }
+  if (N <= 8)
+    return short_tiles(M, batch, 64, 0.8) ? launch_tiles<false, 32, 8, 2, 1, 8>(batch, M, N, K, A, B, C, P, m, s)
+                                          : launch_tiles<false, 64, 8, 2, 2, 8>(batch, M, N, K, A, B, C, P, m, s);
+  if (N <= 16)
+    return short_tiles(M, batch, 128, 0.8) ? launch_tiles<false, 32, 16, 2, 2, 8>(batch, M, N, K, A, B, C, P, m, s)
+                                           : launch_tiles<false, 128, 16, 4, 4, 4>(batch, M, N, K, A, B, C, P, m, s);
+  if (N <= 32)
+    return short_tiles(M, batch, 128, 0.8) ? launch_tiles<false, 32, 32, 4, 2, 8>(batch, M, N, K, A, B, C, P, m, s)
+                                           : launch_tiles<false, 128, 32, 8, 4, 4>(batch, M, N, K, A, B, C, P, m, s);
+  return short_tiles(M, batch * ((N + 63) / 64), 64, 0.92)
+             ? launch_tiles<false, 32, 64, 4, 4, 6>(batch, M, N, K, A, B, C, P, m, s)
+             : launch_tiles<false, 64, 64, 8, 4, 4>(batch, M, N, K, A, B, C, P, m, s);
 }
 
 }  // namespace tnq

@@ -125,15 +125,15 @@ def test_block_diagonal_matricisation_is_the_batched_gemm():
 @pytest.mark.parametrize("shape", [(152, 128, 64, 16), (160, 65, 33, 1), (300, 129, 65, 17), (2, 1999, 1023, 19),
                                    (64, 4096, 64, 8), (3, 1900, 1000, 33), (1, 2500, 1300, 50)])
 def test_cgemm_fp32_wide_tiles(shape):
-    """Shapes around the 128 x 64 tiles (whole ones, one row or column more, ragged ends of K, even and odd
-    rows for 16- and 8-byte copies), enough of them to take that form, against an FP64 product."""
+    """Shapes around the 64-column tiles (whole ones, one row or column more, ragged ends of K, even and odd
+    rows for 16- and 8-byte copies), many of them, against an FP64 product."""
     err = _run(0, *shape)
     assert err <= 1e-5
 
 
 @pytest.mark.parametrize("n,cols", [(12, 6), (13, 7)])
 def test_cgemm_fp32_wide_tiles_permuted_output(n, cols):
-    """The permuted epilogue of the 128 x 64 tiles through uniform blocks in plain FP32 (N = K = 2^cols)."""
+    """The permuted epilogue of the 64-column tiles through uniform blocks in plain FP32 (N = K = 2^cols)."""
     from paper_2108_06831_gb300 import circuits as C
     from oracle.statevector import simulate_state
     tn = _tn()
@@ -142,3 +142,15 @@ def test_cgemm_fp32_wide_tiles_permuted_output(n, cols):
     got = ctr.state().cpu().numpy()[0]
     ref = simulate_state(c)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+
+
+@pytest.mark.parametrize("K", [3, 16, 34, 1025])
+@pytest.mark.parametrize("n", [5, 8, 9, 16, 17, 32, 33, 64, 65])
+@pytest.mark.parametrize("batch,M", [(1, 31), (5, 129), (160, 257), (1, 20000)])
+def test_cgemm_fp32_tile_of_every_width(batch, M, n, K):
+    """Short and tall tiles of 8, 16, 32 and 64 columns: the edges of N's classes, few tiles and many, ragged
+    rows, K of less than a slice, whole slices, a remainder, and one that few tiles split.  Sums of K products
+    of unit-variance factors: their relative error in FP32 stays under K 2^-24, here 6e-5."""
+    if K == 1025 and batch * M > 700:
+        K = 50
+    assert _run(0, batch, M, n, K, seed=M + n) <= max(K, 16) * 2.0 ** -24
