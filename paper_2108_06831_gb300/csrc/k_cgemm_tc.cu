@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgemm_tc(const __grid_constant_
 // The first split_warps: A split; then one for TMA, one for TMEM allocation and MMA issue, and four for the
 // epilogue (warp w owns TMEM lanes 32 (w mod 4)..+31).
 // Warps of the A split: four for TF32; eight for BF16, whose split reads, converts and writes three times
-// as much work per element (batch 64, 32768 x 64 x 64: 510 us with four, 444 with eight; TF32 399 and 403).
+// as much work per element (batch 64, 32768 x 64 x 64: 498 us with four, 462 with eight; TF32 399 and 403).
 template <int PREC>
 constexpr int split_warps() { return PREC == PREC_TF32 ? 4 : 8; }
 template <int PREC>
@@ -454,12 +454,28 @@ constexpr int kStreamMaxKTiles = 8;  // a single leading accumulator per tile st
 // the writes (lanes = rows) and the reads (lanes = bits 1-5 of u) of each half warp fall in distinct
 // banks.  Loads of index tables and bank conflicts of a padded staging were 1500 of the 4100 shared-
 // memory wavefronts of a tile, on a kernel bound by them.
+enum { kStaged = 0, kDirectCols = 1, kDirectRows = 2 };
 struct ChunkMap {
   int row_swz[5];   // S of each row bit
   int s[9];
   long long g[9];
   int pairs;        // u and u + 1 are adjacent in memory
+  // Written back from the registers instead, where a store of the warp covers runs of at least 128 bytes
+  // so (64-byte runs filled by two stores for kDirectCols with column bit 2 below the row bits).
+  // kDirectCols: column bits 0 and 1 are the lowest stored bits and row bits come next, a lane stores four
+  // columns of its row, 32 bytes.  kDirectRows: row bits 0-3 are the lowest, a lane stores single columns.
+  // Staging was 128 of the 900 KB that a tile moves through the shared-memory data pipe, which bounds this
+  // kernel.  Batch 64, 32768 x 64 x 64 stored as the next merge reads it (column bits 0-2, the row bits, then
+  // the others): 437 -> 386 us.  Row-major rows, 512 bytes apart, are staged: 399 us, 496 from registers.
+  int direct;
+  long long row_g[5], col_g[6];  // stored offsets of the row and column bits (of the chunk, and of the tile's chunks)
 };
+// 32 bytes (a whole sector) in one store
+__device__ __forceinline__ void store8(float2 *p, const float *v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
 
 // Split of one A stage from FP32 into three BF16 parts, in place: the FP32 tile is two 128-byte
 // boxes (K elements 32j..32j+31 of every row, 16-byte chunks swizzled by row mod 8); part p is a
@@ -678,11 +694,20 @@ __global__ void __launch_bounds__(stream_threads<PREC>(), 1)
       if ((lane >> k) & 1) {
         wr ^= (16 << k) ^ cm.row_swz[k];
         rd ^= cm.s[k + 1];
-        go += cm.g[k + 1];
+        go += cm.direct ? cm.row_g[k] : cm.g[k + 1];
       }
     long long li = 0;
     for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x, ++li) {
       const int ab = (int)(li & 1);
+      // the tile's stored offset, while its accumulators are still being summed (found per chunk and after the
+      // wait, it was in the way of the tile's other work: 24-qubit blocks of 64 x 64 in split BF16 2375 us, so
+      // 1824; 3xTF32 1629 and 1556)
+      int nt, mt, bz;
+      decode(t, nt, mt, bz);
+      const long long row0 = (long long)bz * M + (long long)mt * BM + q * 32;  // the warp's first row
+      float2 *Ct = reinterpret_cast<float2 *>(C) + go +
+                   (om.identity ? row0 * (N2 / 2) + nt * (BN / 2)
+                                : map_bits(om, (row0 << lgn) | ((long long)nt * (BN / 2)), 0));
       bool have = mbar_wait(&acc_full[ab], (uint32_t)((li / 2) & 1), status);
       have = __all_sync(0xFFFFFFFFu, have);
       if (!have) {
@@ -690,24 +715,36 @@ __global__ void __launch_bounds__(stream_threads<PREC>(), 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      int nt, mt, bz;
-      decode(t, nt, mt, bz);
-      const long long row0 = (long long)bz * M + (long long)mt * BM + q * 32;  // the warp's first row
       const uint32_t base = tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * 2 * BN);
       for (int c = 0; c < BN; c += 32) {
         uint32_t r[32], e[32];
         tmem_ld32(base + BN + c, e);  // corrections
         tmem_ld32(base + c, r);       // leading product
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        float2 *C2 = Ct + ((c & 32) ? cm.col_g[4] : 0) + ((c & 64) ? cm.col_g[5] : 0);
+        if (cm.direct == kDirectRows) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            C2[((k & 1) ? cm.col_g[0] : 0) + ((k & 2) ? cm.col_g[1] : 0) + ((k & 4) ? cm.col_g[2] : 0) +
+               ((k & 8) ? cm.col_g[3] : 0)] = make_float2(__uint_as_float(e[2 * k]) + __uint_as_float(r[2 * k]),
+                                                          __uint_as_float(e[2 * k + 1]) + __uint_as_float(r[2 * k + 1]));
+          continue;
+        }
+        if (cm.direct == kDirectCols) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(e[8 * k + i]) + __uint_as_float(r[8 * k + i]);
+            store8(C2 + ((k & 1) ? cm.col_g[2] : 0) + ((k & 2) ? cm.col_g[3] : 0), v);
+          }
+          continue;
+        }
 #pragma unroll
         for (int k = 0; k < 16; ++k)
           stg[wr ^ k] = make_float2(__uint_as_float(e[2 * k]) + __uint_as_float(r[2 * k]),
                                     __uint_as_float(e[2 * k + 1]) + __uint_as_float(r[2 * k + 1]));
         __syncwarp();
-        // stored offset of everything but the chunk's local bits
-        float2 *C2 = reinterpret_cast<float2 *>(C) + go +
-                     (om.identity ? row0 * (N2 / 2) + nt * (BN / 2) + c / 2
-                                  : map_bits(om, (row0 << lgn) | ((long long)nt * (BN / 2) + c / 2), 0));
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
           const int at = rd ^ ((it & 1) ? cm.s[6] : 0) ^ ((it & 2) ? cm.s[7] : 0) ^ ((it & 4) ? cm.s[8] : 0);
@@ -749,7 +786,7 @@ __global__ void __launch_bounds__(stream_threads<PREC>(), 1)
 }
 
 // The chunk's write-back for columns lgn (log2, with a permuted output) or N complex columns (row-major).
-void chunk_map(ChunkMap &cm, const OutMap &om, long long N) {
+void chunk_map(ChunkMap &cm, const OutMap &om, long long N, const void *C) {
   std::memset(&cm, 0, sizeof(cm));
   int lgn = 0, order[9];
   long long off[9];  // stored offset of local bit b: b < 4 column, else row
@@ -758,7 +795,9 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N) {
     order[b] = b;
     if (om.identity) off[b] = b < 4 ? 1ll << b : N << (b - 4);
     else off[b] = 1ll << (b < 4 ? om.pos[b] : om.pos[lgn + b - 4]);
+    (b < 4 ? cm.col_g[b] : cm.row_g[b - 4]) = off[b];
   }
+  for (int b = 4; b < kColBits; ++b) cm.col_g[b] = 1ll << (om.identity ? b : om.pos[b]);
   std::sort(order, order + 9, [&](int x, int y) { return off[x] < off[y]; });
   // S: the row bits read by a half warp (bits 1-4 of u) take the column bits it does not read; the
   // other row bits among the first four, the lanes of a write, take what is left of the column bits
@@ -786,6 +825,8 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N) {
     cm.g[k] = off[b];
   }
   cm.pairs = off[order[0]] == 1;
+  if (off[0] == 1 && off[1] == 2 && order[3] >= 4 && (uintptr_t)C % 32 == 0) cm.direct = kDirectCols;
+  if (off[4] == 1 && off[5] == 2 && off[6] == 4 && off[7] == 8) cm.direct = kDirectRows;
 }
 
 // ------------------------------------------------------------------------------ prep kernels
@@ -949,7 +990,7 @@ cudaError_t run_tc(long long batch, long long M, long long N, long long K, const
       const long long total = (long long)tiles_n * tiles_m * batch;
       const long long grid = std::min<long long>(total, num_sms());
       ChunkMap cm;
-      chunk_map(cm, om, N);
+      chunk_map(cm, om, N, C);
       return launch_pdl(k_cgemm_tc_stream<PREC>, dim3((unsigned)grid), dim3(stream_threads<PREC>()), smem, s, maps, k_tiles,
                         tiles_n, tiles_m, total, M, 2 * N, reinterpret_cast<float *>(C),
                         static_cast<int *>(status_word_ptr()), om, cm);
