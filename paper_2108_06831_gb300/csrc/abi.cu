@@ -185,7 +185,7 @@ tn_status build_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, s
   const tn_circuit fwd_circ = push_phases(fuse ? fuse_pairs(*c, p->fused) : *c, p->fused);
   for (const TnGate &g : fwd_circ.gates) p->n_fused += g.kind == KIND_F2 ? 1 : 0;
   tn_status st = build_pass_plan(fwd_circ, p->T, p->K, false, p->slots, p->fwd, err);
-  // the adjoint sweep stages two tiles (psi, lambda), double-buffered: at most 2^11 amplitudes each
+  // the adjoint sweep stages two tiles (psi, lambda): at most 2^11 amplitudes each
   const int T_bwd = std::min(p->T, 11);
   if (st == TN_OK && o.target == TN_TARGET_EXPECTATION)
     st = build_pass_plan(*c, T_bwd, std::min(T_bwd, 4), true, p->slots, p->bwd, err);

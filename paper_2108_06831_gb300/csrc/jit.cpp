@@ -816,7 +816,7 @@ std::string rename_array(const std::string &code, const char *to) {
   return out;
 }
 
-// Adjoint-sweep pass: psi and lambda tiles double-buffered in shared memory, every op
+// Adjoint-sweep pass: psi and lambda tiles in shared memory between phases, every op
 // applied (conjugate-transposed) to both, derivative dots accumulated per slot.
 std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, int *threads_out,
                          size_t *smem_out) {
@@ -1224,10 +1224,9 @@ tn_status jit_build(tn_plan &p, const std::vector<int> &op_kind, bool backward, 
     }
     kers[i] = k;
   }
-  {
+  if (backward) {
     // resident CTAs per SM of each pass kernel, queried once here (not per launch)
-    std::vector<int> &grid = backward ? p.jit_bwd_grid : p.jit_grid;
-    grid.assign(np, 1);
+    p.jit_bwd_grid.assign(np, 1);
     for (size_t i = 0; i < np; ++i) {
       int per_sm = 0;
       cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)kers[i], threads[i], smem[i]);
@@ -1235,7 +1234,7 @@ tn_status jit_build(tn_plan &p, const std::vector<int> &op_kind, bool backward, 
         err = std::string("occupancy of a generated kernel: ") + cudaGetErrorString(e);
         return TN_ERR_CUDA;
       }
-      grid[i] = per_sm < 1 ? 1 : per_sm;
+      p.jit_bwd_grid[i] = per_sm < 1 ? 1 : per_sm;
     }
   }
   if (!backward) {
@@ -1260,7 +1259,6 @@ tn_status jit_build(tn_plan &p, const std::vector<int> &op_kind, bool backward, 
 }
 
 void jit_release(tn_plan &p) {
-  p.jit_grid.clear();
   p.jit_bwd_grid.clear();
   p.jit_cm_ptr.clear();
   p.jit_cm_bytes.clear();

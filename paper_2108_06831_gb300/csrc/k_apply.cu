@@ -7,8 +7,9 @@
 // shared memory with coalesced 128-bit loads (the low four index bits are always inside
 // the tile, so every global access is a 128-byte run), runs the pass's phases (each
 // maps K tile bits to registers and applies its ops there) and writes the tile back.
-// Tiles are independent, so the grid is persistent: one wave of CTAs sized from the
-// occupancy calculator, striding over batch x 2^(N-T) tiles.
+// Tiles are independent, so the grid of this interpreting form is persistent: one wave of CTAs sized
+// from the occupancy calculator, striding over batch x 2^(N-T) tiles (the generated form runs one tile
+// per CTA).
 #include <algorithm>
 
 #include "apply_common.cuh"

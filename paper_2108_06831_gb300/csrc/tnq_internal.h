@@ -23,6 +23,7 @@ constexpr int kMaxQubits = 34;   // 2^34 complex64 = 128 GiB, the largest state 
 constexpr int kMaxTile = 13;     // qubits per on-chip tile (2^13 complex64 = 64 KiB of shared memory)
 constexpr int kLowBits = 4;      // the lowest bits always inside a tile: runs of 16 amplitudes = 128 B
 constexpr int kMaxReg = 4;       // register qubits per thread and phase (2^4 amplitudes)
+constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pass of the adjoint sweep
 // Small states: with 16 amplitudes a thread they give an SM too few warps to hide a pass's latency (every
 // gate is a chain of dependent instructions, every phase a barrier).  Below kLeanWarps warps per SM the
 // forward passes run from a plan of kLeanReg register qubits (four amplitudes a thread; one qubit more
@@ -35,7 +36,6 @@ constexpr int kConstMinQubits = 19;  // parameterised circuits, batch 1: constan
 constexpr double kLeanWarps = 8.0;
 constexpr double kLeanGates = 24.0;
 constexpr int kLeanReg = 2;
-constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pass of the adjoint sweep
 
 // ---------------------------------------------------------------------------------------
 // Register-level operations of the fused gate-apply kernel.
@@ -489,7 +489,7 @@ struct tn_plan {
   // plan-specialised forward kernels (generated; empty when the interpreting kernel runs)
   std::vector<cudaLibrary_t> jit_libs;
   std::vector<cudaKernel_t> jit_kernels;
-  std::vector<int> jit_threads, jit_grid;
+  std::vector<int> jit_threads;
   std::vector<size_t> jit_smem;
   std::vector<void *> jit_cm_ptr;    // per forward pass: device address of its __constant__ matrix table
   std::vector<size_t> jit_cm_bytes;  //   and the bytes the pass reads (copied before its launch)

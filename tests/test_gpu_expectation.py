@@ -197,3 +197,32 @@ def test_pauli_sums_over_tile_sizes(n):
         ref = OB.expectation(c, H, params[b])
         assert abs(direct[b] - ref) <= bound
         assert abs(e[b].item() - ref) <= bound
+
+
+@pytest.mark.parametrize("n,tile", [(2, 0), (5, 0), (8, 0), (9, 6), (10, 7), (11, 8)])
+def test_gradients_of_every_parameterised_gate(n, tile):
+    """Gates of one, two-qubit and three angles in mixed order on every qubit: the dots of a phase come in
+    groups of every size, first and last phases with and without the tile's lowest bits in the registers."""
+    from oracle import gradients as GR
+    from oracle import observables as OB
+    tn = _tn()
+    rng = np.random.default_rng(17 * n + tile)
+    gates, at = [], 0
+    for _ in range(5 * n):
+        kind = ["RX", "RY", "RZ", "U3", "U3", "CP", "CZ", "CNOT"][int(rng.integers(0, 8))]
+        arity, angles = C.GATE_ARITY[kind]
+        qs = tuple(int(q) for q in rng.choice(n, size=arity, replace=False))
+        gates.append(C.Gate(kind, qs, (0.0,) * angles, at if angles else -1))
+        at += angles
+    c = C.Circuit(n, gates, n_params=at)
+    H = C.random_pauli_sum(n, 12, 5 + n)
+    params = rng.uniform(0, 2 * np.pi, size=(2, at))
+    ctr = tn.Contractor(c, target=tn.TARGET_EXPECTATION, batch=2, tile_qubits=tile)
+    E, G = ctr.expectation_value_and_grad(tn.Observable(H), _dev(params))
+    torch.cuda.synchronize()
+    assert tn.sync_status() == tn.OK
+    for b in range(2):
+        Eref = OB.expectation(c, H, params[b])
+        assert abs(float(E[b]) - Eref) <= 1e-4 * max(1.0, abs(Eref))
+        gref = GR.param_shift_grad(c, H, params[b])
+        assert np.linalg.norm(G[b].cpu().numpy() - gref) / max(np.linalg.norm(gref), 1e-3) <= 1e-4

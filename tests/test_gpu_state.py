@@ -251,3 +251,37 @@ def test_small_states_take_few_amplitudes_per_thread(n, depth, batch, parameteri
         ref = simulate_state(c, None if params is None else params[b])
         assert rel_l2(got[b], ref) <= STATE_TOL
         assert rel_l2(amps[b], ref[xs]) <= STATE_TOL
+
+
+@pytest.mark.parametrize("parameterized", [False, True])
+@pytest.mark.parametrize("n,tile", [(3, 0), (7, 0), (12, 0), (13, 6), (14, 8), (17, 12), (18, 0)])
+def test_runs_of_diagonal_gates(n, tile, parameterized):
+    """Runs of diagonal gates of every kind between mixing gates on single qubits: operands in the registers,
+    in the tile and outside it, both operands of a pair anywhere, runs that end at a mix or at the phase."""
+    from oracle.statevector import simulate_state
+    rng = np.random.default_rng(31 * n + tile)
+    gates, n_params = [C.Gate("H", (q,)) for q in range(n)], 0
+    one, two = ["Z", "S", "SDG", "T", "TDG", "RZ"], ["CZ", "CP"]
+    for _ in range(6):
+        for _ in range(3 * n):
+            if rng.uniform() < 0.6:
+                kind = two[int(rng.integers(0, 2))]
+                qs = tuple(int(q) for q in rng.choice(n, size=2, replace=False))
+            else:
+                kind, qs = one[int(rng.integers(0, len(one)))], (int(rng.integers(0, n)),)
+            angles, at = (), -1
+            if kind in ("RZ", "CP"):
+                angles = (float(rng.uniform(0, 2 * np.pi)),)
+                if parameterized:
+                    at, n_params = n_params, n_params + 1
+            gates.append(C.Gate(kind, qs, angles, at))
+        for q in rng.choice(n, size=2, replace=False):  # one mixed, one mixed under a control
+            gates.append(C.Gate("SX", (int(q),)))
+        a, b = (int(q) for q in rng.choice(n, size=2, replace=False))
+        gates.append(C.Gate("CNOT", (a, b)))
+    c = C.Circuit(n, gates, n_params=n_params)
+    batch = 2 if parameterized else 1
+    params = rng.uniform(0, 2 * np.pi, size=(batch, n_params)) if parameterized else None
+    got = gpu_state(c, params, batch=batch, tile=tile)
+    for b in range(batch):
+        assert rel_l2(got[b], simulate_state(c, None if params is None else params[b])) <= STATE_TOL
