@@ -402,6 +402,63 @@ struct Deferred {
   }
 };
 
+// CNOTs controlled by a bit outside the registers.  Such a gate moves register j to j ^ (1 << target) where
+// the control is 1.  Next to the phase's loads or stores that is an XOR of their shared-memory addresses,
+// in place of a conditional exchange of all registers, and most can be brought there: the translation
+// passes register CNOTs and SWAPs (linear in the bits of j) as another one, X and other such CNOTs as it is,
+// and every op that does not read or mix the bits it moves; the arithmetic on each amplitude and its order
+// stay the same.  Not an op with a parameter derivative, whose dot sums the registers in order.  Only where
+// the loads or stores are to shared memory (can_in, can_out).  20-qubit ansatz, 64 sets: gradients 19.2 ->
+// 18.7 ms; 22-qubit energies, 4 sets: 787 -> 760 us.
+struct Frame {
+  std::string in = "0", out = "0";  // XOR of the addresses, in the phase's swizzled offsets
+  std::vector<bool> drop;           // per op of the phase: absorbed here
+
+  Frame(const std::vector<OpDesc> &ops, const std::vector<int> &op_kind, const PhaseDesc &d, bool can_in, bool can_out)
+      : drop((size_t)(d.op_end - d.op_begin), false) {
+    const int n = d.op_end - d.op_begin;
+    // register translation v past op i; false where it cannot pass
+    auto pass = [&](int i, int &v) {
+      const OpDesc &op = ops[(size_t)(d.op_begin + i)];
+      const int kind = op_kind[(size_t)(d.op_begin + i)];
+      if (op.has_grad) return false;
+      const int a = op.a_kind == SRC_REG ? (v >> op.a_pos) & 1 : 0, b = op.b_kind == SRC_REG ? (v >> op.b_pos) & 1 : 0;
+      switch (op.type) {
+        case OP_G1: return kind == TN_GATE_X || !a;
+        case OP_C1:
+          if (kind != TN_GATE_CNOT) return !a && !((v >> op.b_pos) & 1);
+          v ^= a << op.b_pos;  // controlled from outside the registers: another translation
+          return true;
+        case OP_G2: {
+          const int x = (v >> op.a_pos) & 1, y = (v >> op.b_pos) & 1;
+          if (kind != TN_GATE_SWAP) return !x && !y;
+          if (x != y) v ^= (1 << op.a_pos) | (1 << op.b_pos);
+          return true;
+        }
+        case OP_D1: return !a;
+        case OP_CZ:
+        case OP_DP: return !a && !b;
+      }
+      return false;
+    };
+    auto absorb = [&](int i, bool front, std::string &to) {
+      const OpDesc &op = ops[(size_t)(d.op_begin + i)];
+      if (drop[(size_t)i] || op.type != OP_C1 || op.a_kind == SRC_REG || op.has_grad ||
+          op_kind[(size_t)(d.op_begin + i)] != TN_GATE_CNOT)
+        return;
+      int v = 1 << op.b_pos, off = 0;
+      for (int k = front ? i - 1 : i + 1; k >= 0 && k < n; k += front ? -1 : 1)
+        if (!drop[(size_t)k] && !pass(k, v)) return;
+      for (int r = 0; r < kMaxReg; ++r)
+        if ((v >> r) & 1) off |= 1 << d.reg_pos[r];
+      to += " ^ (-" + cond_expr(op.a_kind, op.a_pos) + " & " + std::to_string(swz_host(off)) + ")";
+      drop[(size_t)i] = true;
+    };
+    for (int i = 0; i < n && can_in; ++i) absorb(i, true, in);
+    for (int i = n; i-- > 0 && can_out;) absorb(i, false, out);
+  }
+};
+
 }  // namespace
 
 // Forward pass kernels read their matrix entries from a per-pass __constant__ table when one
@@ -579,6 +636,8 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
     E.line("      const int tb = " + tb + ";");
     E.line("      const int pb = swz(tb);");
     const bool from_global = first && !pd.init_mode && !load_staged, to_global = last && !store_staged;
+    const Frame frame(p.fwd.ops, op_kind, d, !from_global && !(first && pd.init_mode), !to_global);
+    E.line("      const int pi = pb ^ (" + frame.in + "), po = pb ^ (" + frame.out + ");");
     if (from_global || to_global) E.line("      float2 *const gt = st + (" + gb + ");");
     if (first && pd.init_mode) {
       std::string li = "0";
@@ -600,17 +659,18 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
       ro[j] = swz_host(off[j]);
       if (first && pd.init_mode) snprintf(buf, sizeof buf, "      a[%d] = make_float2(li == %d ? 1.f : 0.f, 0.f);", j, off[j]);
       else if (from_global) snprintf(buf, sizeof buf, "      a[%d] = gt[%lldll];", j, go[j]);
-      else snprintf(buf, sizeof buf, "      a[%d] = sm[pb ^ %d];", j, ro[j]);
+      else snprintf(buf, sizeof buf, "      a[%d] = sm[pi ^ %d];", j, ro[j]);
       E.line(buf);
     }
     Deferred deferred;
     const bool defer = p.opts.target != TN_TARGET_EXPECTATION;
     for (int o = d.op_begin; o < d.op_end; ++o)
-      if (!defer || !deferred.take(E, p.fwd.ops[o], op_kind[o])) emit_op(E, p.fwd.ops[o], op_kind[o]);
+      if (!frame.drop[(size_t)(o - d.op_begin)] && (!defer || !deferred.take(E, p.fwd.ops[o], op_kind[o])))
+        emit_op(E, p.fwd.ops[o], op_kind[o]);
     deferred.flush_all(E);
     for (int j = 0; j < E.R; ++j) {
       if (to_global) snprintf(buf, sizeof buf, "      gt[%lldll] = a[%d];", go[j], j);
-      else snprintf(buf, sizeof buf, "      sm[pb ^ %d] = a[%d];", ro[j], j);
+      else snprintf(buf, sizeof buf, "      sm[po ^ %d] = a[%d];", ro[j], j);
       E.line(buf);
     }
     E.line("    }");
@@ -967,6 +1027,8 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
     E.line("      const int tb = " + tb + ";");
     E.line("      const int pb = swz(tb);");
     const bool from_global = ph == pd.phase_begin && !load_staged, to_global = ph + 1 == pd.phase_end && !store_staged;
+    const Frame frame(p.bwd.ops, op_kind, d, !from_global, !to_global);
+    E.line("      const int pi = pb ^ (" + frame.in + "), po = pb ^ (" + frame.out + ");");
     if (from_global || to_global) {
       std::string gb = "0ll";
       for (int j = 0; j < T - K; ++j) {
@@ -988,7 +1050,7 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
         }
       ro[j] = swz_host(off);
       if (from_global) snprintf(buf, sizeof buf, "      a[%d] = gp[gt + %lldll]; l[%d] = gl[gt + %lldll];", j, go[j], j, go[j]);
-      else snprintf(buf, sizeof buf, "      a[%d] = smp[pb ^ %d]; l[%d] = sml[pb ^ %d];", j, ro[j], j, ro[j]);
+      else snprintf(buf, sizeof buf, "      a[%d] = smp[pi ^ %d]; l[%d] = sml[pi ^ %d];", j, ro[j], j, ro[j]);
       E.line(buf);
     }
     std::vector<PendingDot> dots;
@@ -998,6 +1060,7 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
     };
     for (int o = d.op_begin; o < d.op_end; ++o) {
       const OpDesc &op = p.bwd.ops[o];
+      if (frame.drop[(size_t)(o - d.op_begin)]) continue;
       if (dots.size() + op.n_grad > 4) emit_dot_sums(E, dots, NW);
       Emitter tmp;
       tmp.K = K;
@@ -1018,7 +1081,7 @@ std::string gen_bwd_pass(const tn_plan &p, int pi, const std::vector<int> &op_ki
     emit_dot_sums(E, dots, NW);
     for (int j = 0; j < E.R; ++j) {
       if (to_global) snprintf(buf, sizeof buf, "      gp[gt + %lldll] = a[%d]; gl[gt + %lldll] = l[%d];", go[j], j, go[j], j);
-      else snprintf(buf, sizeof buf, "      smp[pb ^ %d] = a[%d]; sml[pb ^ %d] = l[%d];", ro[j], j, ro[j], j);
+      else snprintf(buf, sizeof buf, "      smp[po ^ %d] = a[%d]; sml[po ^ %d] = l[%d];", ro[j], j, ro[j], j);
       E.line(buf);
     }
     E.line("    }");

@@ -226,3 +226,37 @@ def test_gradients_of_every_parameterised_gate(n, tile):
         assert abs(float(E[b]) - Eref) <= 1e-4 * max(1.0, abs(Eref))
         gref = GR.param_shift_grad(c, H, params[b])
         assert np.linalg.norm(G[b].cpu().numpy() - gref) / max(np.linalg.norm(gref), 1e-3) <= 1e-4
+
+
+@pytest.mark.parametrize("n,tile", [(3, 0), (6, 0), (9, 6), (11, 7), (12, 8)])
+def test_register_permutations_among_mixing_gates(n, tile):
+    """CNOT, SWAP and X runs between diagonal, mixing and parameterised gates: controls in the registers, in the
+    tile and outside it, exchanges that reach a phase's loads or stores and ones that a gate in between stops."""
+    from oracle import gradients as GR
+    from oracle import observables as OB
+    from oracle.statevector import simulate_state
+    tn = _tn()
+    rng = np.random.default_rng(131 * n + tile)
+    gates, at = [], 0
+    for _ in range(14 * n):
+        kind = ["CNOT", "CNOT", "CNOT", "SWAP", "X", "H", "RZ", "RY", "CZ", "T", "CP", "SX"][int(rng.integers(0, 12))]
+        arity, angles = C.GATE_ARITY[kind]
+        qs = tuple(int(q) for q in rng.choice(n, size=arity, replace=False))
+        free = angles and rng.uniform() < 0.3
+        gates.append(C.Gate(kind, qs, tuple(float(x) for x in rng.uniform(0, 2 * np.pi, size=angles)), at if free else -1))
+        at += angles if free else 0
+    c = C.Circuit(n, gates, n_params=at)
+    H = C.random_pauli_sum(n, 9, 3 + n)
+    params = rng.uniform(0, 2 * np.pi, size=(2, at))
+    psi = tn.Contractor(c, target=tn.TARGET_STATE, batch=2, tile_qubits=tile).state(_dev(params)).cpu().numpy()
+    E, G = tn.Contractor(c, target=tn.TARGET_EXPECTATION, batch=2, tile_qubits=tile).expectation_value_and_grad(
+        tn.Observable(H), _dev(params))
+    torch.cuda.synchronize()
+    assert tn.sync_status() == tn.OK
+    for b in range(2):
+        ref = simulate_state(c, params[b])
+        assert np.linalg.norm(psi[b] - ref) / np.linalg.norm(ref) <= 1e-5
+        Eref = OB.expectation(c, H, params[b])
+        assert abs(float(E[b]) - Eref) <= 1e-4 * max(1.0, abs(Eref))
+        gref = GR.param_shift_grad(c, H, params[b])
+        assert np.linalg.norm(G[b].cpu().numpy() - gref) / max(np.linalg.norm(gref), 1e-3) <= 1e-4
