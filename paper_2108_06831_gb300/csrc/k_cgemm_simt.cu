@@ -19,12 +19,44 @@ namespace {
 
 constexpr int kThreads = 128;  // of a tile's CTA
 
-// An output map with the tables of its permuted epilogue for one tile shape.
+// An output map as runs: the natural index's bits lo..lo + len - 1 are stored at pos..pos + len - 1.
+struct MapRuns {
+  int n;
+  struct {
+    int lo, len, pos;
+  } run[64];
+};
+MapRuns runs_of(const OutMap &om) {
+  MapRuns m;
+  std::memset(&m, 0, sizeof(m));
+  for (int i = 0; i < om.nbits; ++i) {
+    if (i > 0 && om.pos[i] == om.pos[i - 1] + 1) {
+      ++m.run[m.n - 1].len;
+    } else {
+      m.run[m.n].lo = i;
+      m.run[m.n].len = 1;
+      m.run[m.n++].pos = om.pos[i];
+    }
+  }
+  if (om.identity) m.n = 1, m.run[0].lo = m.run[0].pos = 0, m.run[0].len = 62;
+  return m;
+}
+__device__ __forceinline__ long long map_runs(const MapRuns &m, long long f) {
+  long long r = 0;
+  for (int i = 0; i < m.n; ++i) r += ((f >> m.run[i].lo) & ((1ll << m.run[i].len) - 1)) << m.run[i].pos;
+  return r;
+}
+
+// An output map with its permuted epilogue for one tile shape.  The tile's valid local bits are enumerated
+// by increasing stored position as the bits of u: s[k] and g[k] are the staging and stored offsets of u's
+// bit k.
+constexpr int kTileBits = 12;
 struct StagedMap {
-  OutMap map;
-  int lgn, L, nlo, pairs;
-  int s_lo[64], s_hi[64];        // staging offsets (complex)
-  long long g_lo[64], g_hi[64];  // stored offsets (complex)
+  int identity;
+  int lgn, L, pairs;
+  int s[kTileBits];
+  long long g[kTileBits];
+  MapRuns runs;
 };
 void build_staged(StagedMap &sm, const OutMap &om, long long M, long long N, int BM, int BN);
 
@@ -41,35 +73,40 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Permuted output: the tile staged in shared memory (smem, written by the caller, not yet synchronised)
-// goes back in stored-index order, u -> (staging offset, stored offset) from the host-built tables
-// (copied to shared memory: lanes index them divergently).
+// goes back in stored-index order, two elements of u a thread and step.  A thread's offsets are sums over
+// the bits of its index, found once, and of the step; tables of them in shared memory took six loads for
+// every two elements, and a loop over all bits of the map for the tile's own offset (f: its natural index)
+// as many instructions as a tenth of an 8-column tile's.
 template <int THREADS>
-__device__ __forceinline__ void store_staged(const float2 *smem, float2 *__restrict__ C, long long gbase,
+__device__ __forceinline__ void store_staged(const float2 *smem, float2 *__restrict__ C, long long f,
                                              const StagedMap &om) {
-  __shared__ int s_lo[64], s_hi[64];
-  __shared__ long long g_lo[64], g_hi[64];
-  const int L = om.L, nlo = om.nlo, lo_mask = (1 << om.nlo) - 1;
-  if (threadIdx.x < 64) {
-    s_lo[threadIdx.x] = om.s_lo[threadIdx.x];
-    g_lo[threadIdx.x] = om.g_lo[threadIdx.x];
-  }
-  const int hi = THREADS - 1 - (int)threadIdx.x;  // the other end of the CTA
-  if (hi < 1 << (L - nlo)) {
-    s_hi[hi] = om.s_hi[hi];
-    g_hi[hi] = om.g_hi[hi];
-  }
+  constexpr int kLane = THREADS == 128 ? 7 : -1;
+  static_assert(kLane > 0, "bits of the thread index");
+  float2 *c = C + map_runs(om.runs, f);
+  int at = 0;
+#pragma unroll
+  for (int k = 0; k < kLane; ++k)
+    if ((threadIdx.x >> k) & 1) at += om.s[k + 1], c += om.g[k + 1];
   __syncthreads();
-  if (L == 0) {
-    if (threadIdx.x == 0) C[gbase] = smem[0];
-  } else if (om.pairs) {  // u, u + 1 adjacent in memory: 16-byte stores
-    for (int u = 2 * threadIdx.x; u < (1 << L); u += 2 * THREADS) {
-      const float2 x0 = smem[s_lo[u & lo_mask] + s_hi[u >> nlo]];
-      const float2 x1 = smem[s_lo[(u + 1) & lo_mask] + s_hi[(u + 1) >> nlo]];
-      *reinterpret_cast<float4 *>(C + gbase + g_lo[u & lo_mask] + g_hi[u >> nlo]) = make_float4(x0.x, x0.y, x1.x, x1.y);
+  if (om.L == 0) {
+    if (threadIdx.x == 0) c[0] = smem[0];
+    return;
+  }
+  if (threadIdx.x >> (om.L - 1)) return;  // a tile of fewer than two elements per thread
+  const int steps = om.L > kLane + 1 ? 1 << (om.L - kLane - 1) : 1;
+  for (int it = 0; it < steps; ++it) {
+    int s = at;
+    float2 *dst = c;
+#pragma unroll
+    for (int k = 0; k < kTileBits - kLane - 1; ++k)
+      if ((it >> k) & 1) s += om.s[kLane + 1 + k], dst += om.g[kLane + 1 + k];
+    const float2 x0 = smem[s], x1 = smem[s + om.s[0]];
+    if (om.pairs) {  // adjacent in memory
+      *reinterpret_cast<float4 *>(dst) = make_float4(x0.x, x0.y, x1.x, x1.y);
+    } else {
+      dst[0] = x0;
+      dst[om.g[0]] = x1;
     }
-  } else {
-    for (int u = threadIdx.x; u < (1 << L); u += THREADS)
-      C[gbase + g_lo[u & lo_mask] + g_hi[u >> nlo]] = smem[s_lo[u & lo_mask] + s_hi[u >> nlo]];
   }
 }
 
@@ -106,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_cgemm_fp32(long long M, long
                                                             float2 *__restrict__ C, float2 *__restrict__ P,
                                                             const __grid_constant__ StagedMap om) {
   static_assert((BM / TM) * (BN / TN) == kThreads, "one thread per TM x TN block");
-  static_assert(BM * BN <= 1 << 12, "StagedMap covers a tile");
+  static_assert(BM * BN <= 1 << kTileBits, "StagedMap covers a tile");
   constexpr int NX = BN / TN, NY = BM / TM, kSlice = (BM + BN) * kLd;
   extern __shared__ __align__(16) float2 smem[];
   pdl_wait();
@@ -174,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_cgemm_fp32(long long M, long
       }
     }
   }
-  if (SPLIT || om.map.identity) {
+  if (SPLIT || om.identity) {
     float2 *O = SPLIT ? P + ((long long)blockIdx.y * gridDim.z + b) * M * N : C + b * M * N;
 #pragma unroll
     for (int i = 0; i < TM; ++i)
@@ -189,7 +226,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_cgemm_fp32(long long M, long
     for (int i = 0; i < TM; ++i)
 #pragma unroll
       for (int j = 0; j < TN; ++j) smem[(ty + NY * i) * (BN + 1) + tx + NX * j] = acc[i][j];
-    store_staged<kThreads>(smem, C, map_bits(om.map, ((b * M + m0) << om.lgn) | n0, 0), om);
+    store_staged<kThreads>(smem, C, ((b * M + m0) << om.lgn) | n0, om);
   }
 }
 
@@ -200,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_cgemm_fp32(long long M, long
 // multiply-adds), so both give the same bits.
 __global__ void __launch_bounds__(256) k_cgemm_small(long long M, long long N, long long K, long long total,
                                                      const float2 *__restrict__ A, const float2 *__restrict__ B,
-                                                     float2 *__restrict__ C, const __grid_constant__ OutMap om) {
+                                                     float2 *__restrict__ C, const __grid_constant__ MapRuns om) {
   pdl_wait();
   pdl_trigger();
   for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < total;
@@ -217,7 +254,7 @@ __global__ void __launch_bounds__(256) k_cgemm_small(long long M, long long N, l
       acc.y = fmaf(x.x, y.y, acc.y);
       acc.y = fmaf(x.y, y.x, acc.y);
     }
-    C[om.identity ? f : map_bits(om, f, 0)] = acc;
+    C[map_runs(om, f)] = acc;
   }
 }
 constexpr long long kSmallWork = 1ll << 18;
@@ -271,40 +308,28 @@ __global__ void k_splitk_reduce_few(const float2 *__restrict__ P, int splits, lo
   }
 }
 
-// Tables of the permuted epilogue for one tile shape (built on the host once per launch).
-// The tile's valid local bits (vc column bits, then vr row bits) are enumerated by increasing
-// stored position; u's low nlo bits and high L - nlo bits index the tables.
+// The permuted epilogue for one tile shape (built on the host once per launch): the tile's valid local
+// bits are vc column bits, then vr row bits.
 void build_staged(StagedMap &sm, const OutMap &om, long long M, long long N, int BM, int BN) {
-  sm.map = om;
   int lgn = 0, lgm = 0, lbn = 0, lbm = 0;
   while ((1ll << lgn) < N) ++lgn;
   while ((1ll << lgm) < M) ++lgm;
   while ((1 << lbn) < BN) ++lbn;
   while ((1 << lbm) < BM) ++lbm;
-  const int vc = std::min(lbn, lgn), vr = std::min(lbm, lgm), L = vc + vr;
+  const int vc = std::min(lbn, lgn), vr = std::min(lbm, lgm);
   sm.lgn = lgn;
-  sm.L = L;
-  sm.nlo = std::min(L, 6);
-  std::vector<int> order((size_t)L);
-  for (int k = 0; k < L; ++k) order[(size_t)k] = k;
+  sm.L = vc + vr;
+  std::vector<int> order((size_t)sm.L);
+  for (int k = 0; k < sm.L; ++k) order[(size_t)k] = k;
   auto spos = [&](int k) { return (int)(k < vc ? om.pos[k] : om.pos[lgn + k - vc]); };
-  auto sm_of = [&](int k) { return k < vc ? (1 << k) : ((BN + 1) << (k - vc)); };
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return spos(a) < spos(b); });
-  for (int half = 0; half < 2; ++half) {
-    const int nb = half ? L - sm.nlo : sm.nlo, k0 = half ? sm.nlo : 0;
-    for (int u = 0; u < (1 << nb); ++u) {
-      int so = 0;
-      long long go = 0;
-      for (int k = 0; k < nb; ++k)
-        if ((u >> k) & 1) {
-          so += sm_of(order[(size_t)(k0 + k)]);
-          go += 1ll << spos(order[(size_t)(k0 + k)]);
-        }
-      (half ? sm.s_hi : sm.s_lo)[u] = so;
-      (half ? sm.g_hi : sm.g_lo)[u] = go;
-    }
+  for (int k = 0; k < sm.L; ++k) {
+    const int b = order[(size_t)k];
+    sm.s[k] = b < vc ? 1 << b : (BN + 1) << (b - vc);
+    sm.g[k] = 1ll << spos(b);
   }
-  sm.pairs = L > 0 && spos(order[0]) == 0;
+  sm.pairs = sm.L > 0 && sm.g[0] == 1;
+  sm.runs = runs_of(om);
 }
 
 // Tile shape (BM x BN) by which an output of N columns is counted: the split of K and the planner's tile fill.
@@ -343,7 +368,7 @@ cudaError_t launch_tiles(long long batch, long long M, long long N, long long K,
   dim3 grid((unsigned)tiles, (unsigned)splits, (unsigned)batch);
   StagedMap sm;
   std::memset(&sm, 0, sizeof(sm));
-  sm.map = om;
+  sm.identity = om.identity;
   if (!om.identity && !SPLIT) build_staged(sm, om, M, N, BM, BN);
   const bool vec = K % 2 == 0 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
   auto *fn = vec ? k_cgemm_fp32<true, SPLIT, BM, BN, TM, TN, MINB>
@@ -404,7 +429,7 @@ cudaError_t launch_cgemm_fp32(long long batch, long long M, long long N, long lo
   // 13.1, none 22.4)
   if (K <= 64 && ((double)total * (double)K <= (double)kSmallWork || N <= 4)) {
     const long long blocks = std::min<long long>((total + 255) / 256, (long long)num_sms() * 16);
-    return launch_pdl(k_cgemm_small, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, m);
+    return launch_pdl(k_cgemm_small, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, runs_of(m));
   }
   if (P != nullptr) {  // few tiles: the short ones
     if (N <= 8) return launch_tiles<true, 32, 8, 2, 1, 8>(batch, M, N, K, A, B, C, P, m, s);
