@@ -286,6 +286,10 @@ tn_status build_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, s
       }
       if (u != TN_OK) set_error("plan-specialised kernels: %s", jerr.c_str());
     }
+    if (u == TN_OK) {
+      const cudaError_t e = tables_ready();
+      if (e != cudaSuccess) u = cuda_fail(e, "plan tables");
+    }
     if (u != TN_OK) {
       jit_release(*p);
       free_plan_device(p);
@@ -764,6 +768,7 @@ tn_status tn_build_observable(int32_t n_qubits, const tn_pauli_sum *H, tn_observ
   }
   tn_status u = upload(o->terms, &o->d_terms);
   if (u == TN_OK) u = upload(o->passes, &o->d_passes);
+  if (u == TN_OK && (e = tables_ready()) != cudaSuccess) u = cuda_fail(e, "observable tables");
   if (u != TN_OK) {
     cudaFree(o->d_terms);
     cudaFree(o->d_passes);

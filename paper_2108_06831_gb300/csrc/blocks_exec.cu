@@ -141,8 +141,8 @@ tn_status upload_blocks(BlockPlan &bp, bool host_only, bool param_dependent, std
     const size_t mbytes = (size_t)nb * bp.batch * D * D * sizeof(float2);
     e = cudaMalloc((void **)&bp.d_fixed_mats, mbytes);
     if (e == cudaSuccess) e = build_block_mats(bp, nullptr, 0, bp.d_fixed_mats, 0);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
+  if (e == cudaSuccess) e = tables_ready();
   if (e != cudaSuccess) {
     err = std::string("block tables: ") + cudaGetErrorString(e);
     free_blocks(bp);

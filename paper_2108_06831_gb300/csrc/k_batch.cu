@@ -466,6 +466,7 @@ tn_status batch_build(const tn_plan *const *plans, int n, tn_batch **out) {
   b->n_fused_slots = order_slots_fused_first(all_slots);
   if (!all_slots.empty()) up(all_slots.data(), sizeof(MatSlot) * all_slots.size(), (void **)&b->d_slots);
   if (!all_fused.empty()) up(all_fused.data(), sizeof(FusedMember) * all_fused.size(), (void **)&b->d_fused);
+  if (e == cudaSuccess) e = tables_ready();
   if (e != cudaSuccess) {
     batch_free(b);  // the tables allocated so far, the side streams and their events
     return cuda_fail(e, "batched executor tables");
@@ -544,7 +545,8 @@ int batch_device(const tn_batch *b) { return b->device; }
 
 tn_status batch_test_stall(tn_batch *b, int circ, int pass, long long wait_ns) {
   auto upload = [&](int k) -> cudaError_t {
-    return cudaMemcpy(b->d_tasks + k, &b->h_tasks[(size_t)k], sizeof(BatchTask), cudaMemcpyHostToDevice);
+    const cudaError_t e = cudaMemcpy(b->d_tasks + k, &b->h_tasks[(size_t)k], sizeof(BatchTask), cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? tables_ready() : e;
   };
   // restore the table and the default bound first
   if (b->stalled_task >= 0) {

@@ -228,6 +228,8 @@ cudaError_t launch_zero(void *p, size_t bytes, cudaStream_t s) {
   return cudaMemsetAsync(p, 0, bytes, s);
 }
 
+cudaError_t tables_ready() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 // ---------------------------------------------------------------------------------------
 // Device status word: kernels with bounded waits or finiteness checks record the first
 // failure here (atomicCAS from 0); tn_sync_status reads and clears it.
@@ -249,6 +251,7 @@ cudaError_t read_and_clear_status(int *value, cudaStream_t s) {
   if (v != 0) {
     const int zero = 0;
     e = cudaMemcpyToSymbol(g_tn_status, &zero, sizeof(int));
+    if (e == cudaSuccess) e = tables_ready();
     if (e != cudaSuccess) return e;
   }
   *value = v;

@@ -737,7 +737,7 @@ cudaError_t q428_upload(Q428Plan *p) {
   up(p->phases.data(), sizeof(QPhase) * p->phases.size(), (void **)&p->d_phases);
   up(p->ops.data(), sizeof(QOp) * p->ops.size(), (void **)&p->d_ops);
   up(p->mats.data(), sizeof(int32_t) * p->mats.size(), (void **)&p->d_mats);
-  return e;
+  return e == cudaSuccess ? tables_ready() : e;
 }
 
 void q428_free(Q428Plan *p) {

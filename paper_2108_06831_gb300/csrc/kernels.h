@@ -12,6 +12,11 @@ int num_sms();  // SM count of the current device (cached per device)
 // resident per SM.  Rows of ceil(slots / batch) CTAs would leave a few CTAs for a second wave that lasts
 // as long as the first (64 rows of 10 on 608 slots).
 long long grid_per_row(long long n_tiles, long long batch, int per_sm);
+// Ends whatever has copied tables to the device.  The copies run on the legacy stream, and cudaMemcpy may
+// return before the device holds what it copied: a pageable source has only been staged by then, and a copy
+// within the device does not block at all.  Nothing orders a first call on a non-blocking stream after them
+// but this wait.
+cudaError_t tables_ready();
 
 #ifdef __CUDACC__
 // Programmatic dependent launch (short kernels of the network path).  A kernel launched with

@@ -516,6 +516,7 @@ tn_status upload_network(NetPlan &net, std::string &err) {
   if (e == cudaSuccess) e = cudaMalloc(&net.d_outputs, std::max<size_t>(outs.size(), 1) * sizeof(OutDesc));
   if (e == cudaSuccess && !outs.empty())
     e = cudaMemcpy(net.d_outputs, outs.data(), outs.size() * sizeof(OutDesc), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = tables_ready();
   if (e != cudaSuccess) {
     err = std::string("network tables: ") + cudaGetErrorString(e);
     return TN_ERR_OOM;
