@@ -327,18 +327,26 @@ void emit_op(Emitter &E, const OpDesc &op, int kind) {
 // ops commute, and bits outside the registers are not mixed within a phase.  A QFT's ladder of
 // controlled phases then costs each amplitude one multiplication per register qubit instead of one per
 // gate: 22 qubits 74 -> 53 us, 24 qubits 300 -> 197.  Expectation plans keep the op-by-op form, whose FP32 roundings their
-// FP64 energies and gradients show.
+// FP64 energies and gradients show.  Only phases (entries of modulus one) are deferred: products of a MAT1's
+// entries could leave the FP32 range where the amplitude they scale would not.  A thread whose conditions
+// were all false leaves its amplitudes alone (t<r>): one driven to infinity would become NaN times (1, 0).
 struct Deferred {
   bool q[5] = {false, false, false, false, false}, q_decl[5] = {false, false, false, false, false};
   bool s[5] = {false, false, false, false, false}, s_decl[5] = {false, false, false, false, false};
+  bool always[5] = {false, false, false, false, false};  // q<r> holds a phase whatever the conditions
   static constexpr int kAll = 4;
 
   void phase(Emitter &E, int r, const std::string &cond, const std::string &e, const std::string &other) {
-    const std::string v = "q" + std::to_string(r);
-    if (!q_decl[r]) E.line("float2 " + v + ";");
+    const std::string v = "q" + std::to_string(r), t = "t" + std::to_string(r), one = "make_float2(1.f, 0.f)";
+    if (!q_decl[r]) E.line("float2 " + v + "; unsigned " + t + ";");
     q_decl[r] = true;
+    const bool either = other != one;
+    if (!q[r]) always[r] = false;
+    if (!either) E.line(t + (q[r] ? " |= " : " = ") + cond + ";");
+    else if (!q[r]) E.line(t + " = 1u;");
+    always[r] = always[r] || either;
     if (!q[r]) E.line(v + " = (" + cond + ") ? " + e + " : " + other + ";");
-    else if (other == "make_float2(1.f, 0.f)") E.line("if (" + cond + ") " + v + " = cm(" + v + ", " + e + ");");
+    else if (!either) E.line("if (" + cond + ") " + v + " = cm(" + v + ", " + e + ");");
     else E.line(v + " = cm(" + v + ", (" + cond + ") ? " + e + " : " + other + ");");
     q[r] = true;
   }
@@ -352,14 +360,17 @@ struct Deferred {
   // what is pending on register bit r (kAll: on every amplitude), applied to the registers
   void flush(Emitter &E, int r) {
     const std::string n = std::to_string(r);
-    for (int j = 0; j < E.R && (q[r] || s[r]); ++j) {
-      if (r != kAll && !(j & (1 << r))) continue;
-      const std::string a = "a[" + std::to_string(j) + "]";
-      std::string v = a;
-      if (s[r]) v = "sx(" + v + ", g" + n + ")";
-      if (q[r]) v = "cm(" + v + ", q" + n + ")";
-      E.line(a + " = " + v + ";");
-    }
+    auto each = [&](const std::string &fn, const std::string &by) {
+      for (int j = 0; j < E.R; ++j)
+        if (r == kAll || (j & (1 << r))) {
+          const std::string a = "a[" + std::to_string(j) + "]";
+          E.line("  " + a + " = " + fn + "(" + a + ", " + by + n + ");");
+        }
+    };
+    if (s[r]) each("sx", "g");
+    if (q[r] && !always[r]) E.line("if (t" + n + ") {");
+    if (q[r]) each("cm", "q");
+    if (q[r] && !always[r]) E.line("}");
     q[r] = s[r] = false;
   }
   void flush_all(Emitter &E) {
@@ -375,7 +386,7 @@ struct Deferred {
     const std::string one = "make_float2(1.f, 0.f)";
     switch (op.type) {
       case OP_D1: {
-        if (op.a_kind == SRC_REG) return false;
+        if (op.a_kind == SRC_REG || kind == TN_GATE_MAT1) return false;
         const std::string c = cond_expr(op.a_kind, op.a_pos);
         if (kind == TN_GATE_Z) sign(E, kAll, c);
         else if (kind == KIND_P || kind == TN_GATE_S || kind == TN_GATE_SDG || kind == TN_GATE_T || kind == TN_GATE_TDG)

@@ -285,3 +285,24 @@ def test_runs_of_diagonal_gates(n, tile, parameterized):
     got = gpu_state(c, params, batch=batch, tile=tile)
     for b in range(batch):
         assert rel_l2(got[b], simulate_state(c, None if params is None else params[b])) <= STATE_TOL
+
+
+@pytest.mark.parametrize("n,tile", [(7, 0), (12, 0), (14, 8), (18, 0)])
+def test_diagonal_gates_leave_what_their_condition_excludes(n, tile):
+    """Amplitudes that a MAT1 drove to infinity stay infinite under phases and signs whose condition is false
+    for them (no inf * 0), wherever the condition's bit lies; the others stay exact."""
+    from oracle.statevector import simulate_state
+    tn = _tn()
+    big = float(2.0 ** 100)
+    for q in (0, n // 2, n - 1):
+        h = [C.Gate("H", (k,)) for k in range(n)]
+        scale = [C.Gate("MAT1", (q,), mat=(big, 0, 0, 1))] * 2
+        phases = [C.Gate(kind, (q,)) for kind in ("S", "T", "SDG", "TDG", "Z")]
+        for k in range(n):
+            if k != q:
+                phases += [C.Gate("CP", (q, k), (0.1 + k,)), C.Gate("CZ", (k, q))]
+        ctr = tn.Contractor(C.Circuit(n, h + scale + phases), tile_qubits=tile, fuse=False)
+        got = ctr.state().cpu().numpy()[0].reshape(1 << q, 2, -1)
+        ref = simulate_state(C.Circuit(n, h + phases)).reshape(1 << q, 2, -1)
+        assert np.all(np.isposinf(got[:, 0].real)) and np.all(got[:, 0].imag == 0), q
+        assert rel_l2(got[:, 1], ref[:, 1]) <= STATE_TOL, q
