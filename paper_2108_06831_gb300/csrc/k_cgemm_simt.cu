@@ -19,31 +19,26 @@ namespace {
 
 constexpr int kThreads = 128;  // of a tile's CTA
 
-// An output map as runs: the natural index's bits lo..lo + len - 1 are stored at pos..pos + len - 1.
+// An output map as runs: the natural index's bits lo[i] .. lo[i + 1] - 1 are stored from pos[i] up.  In bytes:
+// it is a parameter of every launch, and the launches are what a network of small merges spends its time on
+// (3 x 6 grid of depth 8, one bitstring, eager calls: 48.5 us with runs of three ints, 772 bytes in all, and 44.5).
 struct MapRuns {
-  int n;
-  struct {
-    int lo, len, pos;
-  } run[64];
+  uint8_t n, lo[64], pos[64];
 };
+static_assert(sizeof(MapRuns) == 129, "small as a kernel parameter");
 MapRuns runs_of(const OutMap &om) {
   MapRuns m;
-  std::memset(&m, 0, sizeof(m));
-  for (int i = 0; i < om.nbits; ++i) {
-    if (i > 0 && om.pos[i] == om.pos[i - 1] + 1) {
-      ++m.run[m.n - 1].len;
-    } else {
-      m.run[m.n].lo = i;
-      m.run[m.n].len = 1;
-      m.run[m.n++].pos = om.pos[i];
-    }
-  }
-  if (om.identity) m.n = 1, m.run[0].lo = m.run[0].pos = 0, m.run[0].len = 62;
+  int n = 0;
+  if (om.identity) m.lo[n] = m.pos[n] = 0, ++n;
+  for (int i = 0; !om.identity && i < om.nbits; ++i)
+    if (i == 0 || om.pos[i] != om.pos[i - 1] + 1) m.lo[n] = (uint8_t)i, m.pos[n] = om.pos[i], ++n;
+  m.n = (uint8_t)n;
+  m.lo[n] = 63;  // a natural index has fewer bits
   return m;
 }
 __device__ __forceinline__ long long map_runs(const MapRuns &m, long long f) {
   long long r = 0;
-  for (int i = 0; i < m.n; ++i) r += ((f >> m.run[i].lo) & ((1ll << m.run[i].len) - 1)) << m.run[i].pos;
+  for (int i = 0; i < m.n; ++i) r += ((f >> m.lo[i]) & ((1ll << (m.lo[i + 1] - m.lo[i])) - 1)) << m.pos[i];
   return r;
 }
 
