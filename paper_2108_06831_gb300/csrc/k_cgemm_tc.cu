@@ -455,11 +455,13 @@ constexpr int kStreamMaxKTiles = 8;  // a single leading accumulator per tile st
 // banks.  Loads of index tables and bank conflicts of a padded staging were 1500 of the 4100 shared-
 // memory wavefronts of a tile, on a kernel bound by them.
 enum { kStaged = 0, kDirectCols = 1, kDirectRows = 2 };
+// (A parameter of every launch: 136 bytes; with all offsets in it, 228, a one-tile call took 10.65 us, 10.45 now.)
 struct ChunkMap {
-  int row_swz[5];   // S of each row bit
-  int s[9];
   long long g[9];
-  int pairs;        // u and u + 1 are adjacent in memory
+  long long chunk_g[2];  // stored offsets of the column bits above the chunk's
+  int s[9];
+  uint8_t row_swz[5];    // S of each row bit
+  bool pairs;            // u and u + 1 are adjacent in memory
   // Written back from the registers instead, where a store of the warp covers runs of at least 128 bytes
   // so (64-byte runs filled by two stores for kDirectCols with column bit 2 below the row bits).
   // kDirectCols: column bits 0 and 1 are the lowest stored bits and row bits come next, a lane stores four
@@ -467,9 +469,11 @@ struct ChunkMap {
   // Staging was 128 of the 900 KB that a tile moves through the shared-memory data pipe, which bounds this
   // kernel.  Batch 64, 32768 x 64 x 64 stored as the next merge reads it (column bits 0-2, the row bits, then
   // the others): 437 -> 386 us.  Row-major rows, 512 bytes apart, are staged: 399 us, 496 from registers.
-  int direct;
-  long long row_g[5], col_g[6];  // stored offsets of the row and column bits (of the chunk, and of the tile's chunks)
+  // Both take the row bits' offsets from g[1] .. g[5], where a staged chunk has its lanes', and the column
+  // bits' from g[0], g[6], g[7] and g[8].
+  uint8_t direct;
 };
+static_assert(sizeof(ChunkMap) == 136, "small as a kernel parameter");
 // 32 bytes (a whole sector) in one store
 __device__ __forceinline__ void store8(float2 *p, const float *v) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
@@ -694,7 +698,7 @@ __global__ void __launch_bounds__(stream_threads<PREC>(), 1)
       if ((lane >> k) & 1) {
         wr ^= (16 << k) ^ cm.row_swz[k];
         rd ^= cm.s[k + 1];
-        go += cm.direct ? cm.row_g[k] : cm.g[k + 1];
+        go += cm.g[k + 1];
       }
     long long li = 0;
     for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x, ++li) {
@@ -721,12 +725,12 @@ __global__ void __launch_bounds__(stream_threads<PREC>(), 1)
         tmem_ld32(base + BN + c, e);  // corrections
         tmem_ld32(base + c, r);       // leading product
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        float2 *C2 = Ct + ((c & 32) ? cm.col_g[4] : 0) + ((c & 64) ? cm.col_g[5] : 0);
+        float2 *C2 = Ct + ((c & 32) ? cm.chunk_g[0] : 0) + ((c & 64) ? cm.chunk_g[1] : 0);
         if (cm.direct == kDirectRows) {
 #pragma unroll
           for (int k = 0; k < 16; ++k)
-            C2[((k & 1) ? cm.col_g[0] : 0) + ((k & 2) ? cm.col_g[1] : 0) + ((k & 4) ? cm.col_g[2] : 0) +
-               ((k & 8) ? cm.col_g[3] : 0)] = make_float2(__uint_as_float(e[2 * k]) + __uint_as_float(r[2 * k]),
+            C2[((k & 1) ? cm.g[0] : 0) + ((k & 2) ? cm.g[6] : 0) + ((k & 4) ? cm.g[7] : 0) +
+               ((k & 8) ? cm.g[8] : 0)] = make_float2(__uint_as_float(e[2 * k]) + __uint_as_float(r[2 * k]),
                                                           __uint_as_float(e[2 * k + 1]) + __uint_as_float(r[2 * k + 1]));
           continue;
         }
@@ -736,7 +740,7 @@ __global__ void __launch_bounds__(stream_threads<PREC>(), 1)
             float v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(e[8 * k + i]) + __uint_as_float(r[8 * k + i]);
-            store8(C2 + ((k & 1) ? cm.col_g[2] : 0) + ((k & 2) ? cm.col_g[3] : 0), v);
+            store8(C2 + ((k & 1) ? cm.g[7] : 0) + ((k & 2) ? cm.g[8] : 0), v);
           }
           continue;
         }
@@ -795,9 +799,8 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N, const void *C) {
     order[b] = b;
     if (om.identity) off[b] = b < 4 ? 1ll << b : N << (b - 4);
     else off[b] = 1ll << (b < 4 ? om.pos[b] : om.pos[lgn + b - 4]);
-    (b < 4 ? cm.col_g[b] : cm.row_g[b - 4]) = off[b];
   }
-  for (int b = 4; b < kColBits; ++b) cm.col_g[b] = 1ll << (om.identity ? b : om.pos[b]);
+  for (int b = 4; b < kColBits; ++b) cm.chunk_g[b - 4] = 1ll << (om.identity ? b : om.pos[b]);
   std::sort(order, order + 9, [&](int x, int y) { return off[x] < off[y]; });
   // S: the row bits read by a half warp (bits 1-4 of u) take the column bits it does not read; the
   // other row bits among the first four, the lanes of a write, take what is left of the column bits
@@ -808,7 +811,7 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N, const void *C) {
   for (int r = 0; r < 5; ++r) {
     if (!row_read[r]) continue;
     while (col_read[next]) ++next;
-    cm.row_swz[r] = 1 << next;
+    cm.row_swz[r] = (uint8_t)(1 << next);
     if (r < 4) taken[next] = true;
     ++next;
   }
@@ -816,7 +819,7 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N, const void *C) {
   for (int r = 0; r < 4; ++r) {
     if (row_read[r]) continue;
     while (taken[next]) ++next;
-    cm.row_swz[r] = 1 << next;
+    cm.row_swz[r] = (uint8_t)(1 << next);
     taken[next] = true;
   }
   for (int k = 0; k < 9; ++k) {
@@ -827,6 +830,10 @@ void chunk_map(ChunkMap &cm, const OutMap &om, long long N, const void *C) {
   cm.pairs = off[order[0]] == 1;
   if (off[0] == 1 && off[1] == 2 && order[3] >= 4 && (uintptr_t)C % 32 == 0) cm.direct = kDirectCols;
   if (off[4] == 1 && off[5] == 2 && off[6] == 4 && off[7] == 8) cm.direct = kDirectRows;
+  if (cm.direct) {
+    for (int k = 0; k < 5; ++k) cm.g[k + 1] = off[k + 4];
+    cm.g[0] = off[0], cm.g[6] = off[1], cm.g[7] = off[2], cm.g[8] = off[3];
+  }
 }
 
 // ------------------------------------------------------------------------------ prep kernels
