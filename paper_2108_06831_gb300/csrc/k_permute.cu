@@ -16,6 +16,7 @@
 // permutations of 27 legs took 414 us (5.2 TB/s), with lo = 6 352 us (6.1 TB/s, 90% of the copy bandwidth).
 // Every mbarrier wait is bounded: on expiry the kernel records TN_ERR_TIMEOUT in the
 // device status word and returns.
+#include <algorithm>
 #include <cstring>
 
 #include "apply_common.cuh"
@@ -27,6 +28,7 @@ namespace {
 
 constexpr int kPermThreads = 256;
 constexpr int kPermStages = 2;
+constexpr int kPermCtas = 6;  // resident per SM, by the registers (40 a thread)
 constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of every mbarrier wait
 
 constexpr int kPermLo = 6;          // low bits: runs of 64 elements = 512 bytes
@@ -281,12 +283,12 @@ cudaError_t launch_permute(int n, const int32_t *perm, long long batch, const fl
   P.n_outer = no;
   P.row_stride = (1 << lo) + 2;
   const size_t smem = (size_t)kPermStages * (1 << P.r) * P.row_stride * sizeof(float2);
-  int per_sm = 0;
   cudaError_t err = ensure_smem(reinterpret_cast<const void *>(k_permute), smem);
-  if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_permute, kPermThreads, smem);
   if (err != cudaSuccess) return err;
-  if (per_sm < 1) per_sm = 1;
   const long long work = (1ll << no) * batch;
+  // resident CTAs per SM: kPermCtas by their registers, fewer by the 228 KB of shared memory (found here: the
+  // occupancy query is several percent of a short call)
+  const long long per_sm = std::max<long long>(1, std::min<long long>(kPermCtas, (228 * 1024) / (long long)(smem + 3072)));
   long long grid = (long long)num_sms() * per_sm;
   if (grid > work) grid = work;
   k_permute<<<(unsigned)grid, kPermThreads, smem, s>>>(P, batch, in, out);
