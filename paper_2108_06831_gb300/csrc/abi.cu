@@ -14,6 +14,7 @@
 #include "network.h"
 #include "blocks.h"
 #include "kernels.h"
+#include "row_grid.h"
 #include "tnq_internal.h"
 
 namespace tnq {
@@ -59,16 +60,7 @@ int num_sms() {
 }
 
 long long grid_per_row(long long n_tiles, long long batch, int per_sm) {
-  const long long slots = (long long)num_sms() * std::max(per_sm, 1);
-  const long long most = std::max<long long>(1, std::min(n_tiles, (4 * slots + batch - 1) / batch));
-  long long best = 1;
-  double best_cost = 0.0;
-  for (long long gx = 1; gx <= most; ++gx) {
-    // tiles of a CTA, and one more for its start and end, times the waves
-    const double cost = (double)((n_tiles + gx - 1) / gx + 1) * (double)((gx * batch + slots - 1) / slots);
-    if (gx == 1 || cost < best_cost) best = gx, best_cost = cost;
-  }
-  return best;
+  return best_row_grid(n_tiles, batch, (long long)num_sms() * std::max(per_sm, 1));
 }
 
 // The dynamic shared-memory limit of a kernel is a per-device function attribute: raise it on

@@ -240,8 +240,9 @@ cudaError_t launch_backward(const tn_plan *p, const float2 *mats, long long mstr
       const int per_sm = i < p->jit_bwd_grid.size() ? p->jit_bwd_grid[i] : 1;  // queried at load time
       cudaError_t e = cudaSuccess;
       const long long n_tiles = 1ll << h.n_outer;
-      // about four tiles per CTA where that is many waves (2 and 4 tiles 20.7 and 20.8 ms on 20 qubits, 64
-      // sets, 16 tiles 21.9, 57 tiles in one wave 23.6: the CTAs of an SM progress unevenly)
+      // About four tiles per CTA where that is the wider grid, many waves (2 and 4 tiles 20.7 and 20.8 ms on 20
+      // qubits, 64 sets, 16 tiles 21.9, 57 tiles in one wave 23.6: the CTAs of an SM progress unevenly); few
+      // tiles fill whole waves.
       const long long gx = std::max(grid_per_row(n_tiles, p->batch, per_sm), n_tiles / 4);
       const float2 *m = mats;
       int np = p->n_params;
