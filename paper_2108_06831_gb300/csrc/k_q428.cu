@@ -742,9 +742,9 @@ cudaError_t q428_upload(Q428Plan *p) {
 
 void q428_free(Q428Plan *p) {
   if (!p) return;
-  cudaFree(p->d_phases);
-  cudaFree(p->d_ops);
-  cudaFree(p->d_mats);
+  // a plan made for the host alone has no tables, and even cudaFree(NULL) would start the runtime
+  for (void *t : {(void *)p->d_phases, (void *)p->d_ops, (void *)p->d_mats})
+    if (t) cudaFree(t);
   delete p;
 }
 

@@ -288,3 +288,31 @@ def test_generated_kernels_compile_without_a_device(tmp_path, monkeypatch):
     assert any("tnq_p" in t for t in srcs) and any("tnq_b" in t for t in srcs)
     assert all("griddepcontrol.wait" in t for t in srcs)  # every pass waits for its predecessor
     assert any("fma.rn.f32x2" in t for t in srcs)
+
+
+def test_host_only_plans_leave_the_driver_alone(tmp_path):
+    """Making, asking and freeing a host-only plan of any kind never loads the driver library (a stand-in for it
+    says so when it is loaded)."""
+    import shutil
+    import subprocess
+    import sys
+    if shutil.which("gcc") is None:
+        pytest.skip("no C compiler")
+    (tmp_path / "cuda.c").write_text(
+        'static void __attribute__((constructor)) loaded(void) {'
+        ' extern int puts(const char *); puts("driver library loaded"); }')
+    subprocess.run(["gcc", "-shared", "-fPIC", "-fno-builtin", "-o", str(tmp_path / "libcuda.so.1"),
+                    str(tmp_path / "cuda.c")], check=True)
+    program = """
+from paper_2108_06831_gb300 import circuits as C, tn
+c = C.brickwork(14, 4, 3)[0]
+for kw in (dict(), dict(target=tn.TARGET_EXPECTATION), dict(q428=True), dict(block_qubits=6),
+           dict(target=tn.TARGET_AMPLITUDES, network_bitstrings=4)):
+    p = tn.Plan(tn.CircuitHandle(c), host_only=True, **kw)
+    p.stats()
+    del p
+print("done")
+"""
+    env = dict(os.environ, LD_LIBRARY_PATH=f"{tmp_path}:{os.environ.get('LD_LIBRARY_PATH', '')}")
+    done = subprocess.run([sys.executable, "-c", program], cwd=ROOT, env=env, capture_output=True, text=True)
+    assert done.stdout.split() == ["done"], done.stdout + done.stderr
