@@ -496,10 +496,11 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
   // then only serves the batched executor's tables and needs no generated kernels.
   double mixing = 0.0;  // gates that mix amplitudes: permutations and diagonal gates are cheap either way
   for (const TnGate &g : c->gates) mixing += lean_weight(g);
-  const bool lean = o.target != TN_TARGET_EXPECTATION && !p->host_only && !(o.flags & TN_PLAN_NO_SPECIALIZE) &&
+  const double sms = p->host_only ? kTargetSms : num_sms();  // a host-only plan is the plan of a GB300
+  const bool lean = o.target != TN_TARGET_EXPECTATION && !(o.flags & TN_PLAN_NO_SPECIALIZE) &&
                     T >= kLowBits + 2 && c->n < kBatchDirectMinQubits && mixing >= kLeanGates &&
                     (c->n_params == 0 || c->n < kFuseMinQubitsParam) &&
-                    std::ldexp((double)o.batch, c->n - 9) < kLeanWarps * (double)num_sms();
+                    std::ldexp((double)o.batch, c->n - 9) < kLeanWarps * sms;
   tn_plan_opts o_main = o;
   if (lean) o_main.flags |= TN_PLAN_NO_SPECIALIZE;
   tn_status st = build_passes(c, o_main, p, err);
@@ -511,7 +512,7 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
     q->n_gates = p->n_gates;
     q->init = p->init;
     q->opts = o;
-    q->host_only = false;
+    q->host_only = p->host_only;
     q->device = -1;
     q->T = T;
     q->K = c->n <= 12 && T <= 12 ? kLeanReg : kLeanReg + 1;  // at most 1024 threads

@@ -33,6 +33,7 @@ constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pas
 // twice the threads, which costs more than the warps gain (16 qubits, 8 sets: 47 against 55 us).
 // Measured: 9 qubits depth 6, one set 20.6 -> 10.4 us; 10 qubits depth 8, 128 sets 26.7 -> 14.4 us.
 constexpr int kConstMinQubits = 19;  // parameterised circuits, batch 1: constant tables from this width on
+constexpr int kTargetSms = 152;      // GB300
 constexpr double kLeanWarps = 8.0;
 constexpr double kLeanGates = 24.0;
 constexpr int kLeanReg = 2;

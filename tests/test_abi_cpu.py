@@ -290,6 +290,27 @@ def test_generated_kernels_compile_without_a_device(tmp_path, monkeypatch):
     assert any("fma.rn.f32x2" in t for t in srcs)
 
 
+def test_small_plans_compile_without_a_device(tmp_path, monkeypatch):
+    """Host-only plans of few warps are the ones that run: two or three register qubits, their kernels generated
+    and compiled (constant and staged tables, one tile and several, runs of diagonal gates)."""
+    tn = _tn()
+    dump = tmp_path / "src"
+    monkeypatch.setenv("TNQ_JIT_COMPILE_CHECK", "1")
+    monkeypatch.setenv("TNQ_JIT_DUMP_DIR", str(dump))
+    monkeypatch.setenv("TNQ_CACHE_DIR", str(tmp_path / "cache"))
+
+    def reg_qubits(circ, **kw):
+        return tn.Plan(tn.CircuitHandle(circ), host_only=True, **kw).stats()["reg_qubits"]
+    nine, fixed = C.brickwork(9, 6, 5, parameterized=True)[0], C.brickwork(14, 4, 5)[0]
+    assert reg_qubits(nine) == 2 and reg_qubits(C.qft(10, 3), target=tn.TARGET_AMPLITUDES) == 4
+    assert reg_qubits(nine, target=tn.TARGET_AMPLITUDES) == 2 and reg_qubits(fixed) == 3
+    assert reg_qubits(nine, batch=1215) == 2 and reg_qubits(nine, batch=1216) == 4  # 8 warps on each of 152 SMs
+    assert reg_qubits(nine, specialize=False) == 4 and reg_qubits(nine, target=tn.TARGET_EXPECTATION) == 4
+    srcs = [f.read_text() for f in dump.glob("*.cu")]
+    for regs in (4, 8, 16):
+        assert any(f"float2 a[{regs}];" in t for t in srcs)
+
+
 def test_host_only_plans_leave_the_driver_alone(tmp_path):
     """Making, asking and freeing a host-only plan of any kind never loads the driver library (a stand-in for it
     says so when it is loaded)."""

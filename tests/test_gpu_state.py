@@ -253,6 +253,16 @@ def test_small_states_take_few_amplitudes_per_thread(n, depth, batch, parameteri
         assert rel_l2(amps[b], ref[xs]) <= STATE_TOL
 
 
+@pytest.mark.parametrize("n,batch,parameterized", [(5, 1, False), (6, 1, True), (9, 1215, True), (9, 1216, True),
+                                                   (13, 1, False), (14, 2, True), (18, 1, False), (19, 1, True)])
+def test_host_only_plans_describe_the_plans_that_run(n, batch, parameterized):
+    tn = _tn()
+    ch = tn.CircuitHandle(C.brickwork(n, 6, n, parameterized=parameterized)[0])
+    host, run = (tn.Plan(ch, batch=batch, host_only=h) for h in (True, False))
+    differ = {k for k, v in run.stats().items() if host.stats()[k] != v}
+    assert differ <= {"specialized"} and host.workspace_bytes == run.workspace_bytes
+
+
 @pytest.mark.parametrize("parameterized", [False, True])
 @pytest.mark.parametrize("n,tile", [(3, 0), (7, 0), (12, 0), (13, 6), (14, 8), (17, 12), (18, 0)])
 def test_runs_of_diagonal_gates(n, tile, parameterized):
