@@ -515,6 +515,9 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
   // blocks; with them three, two when their entries are staged in shared memory (18 qubits, one set: 41 us
   // with two, 66 with three; 24 qubits from constant memory 1195, 1060 and 1122 us with two, three and four)
   int min_blocks = !blocks ? 4 : cmem ? 3 : 2;
+  // These are CTAs of 256 threads: tiles of 13 qubits, 512 threads, would be left 32 or 42 registers and spill
+  // (20-qubit brickwork 56 us with three, 27 with one; 20-qubit energies of two sets 342 with four, 94 with two)
+  if (NTHR > 256) min_blocks = std::max(1, min_blocks * 256 / NTHR);
   if (p.is_lean) min_blocks = std::max(1, std::min(4, 1024 / NTHR));
   if (const char *mb = getenv("TNQ_JIT_MIN_BLOCKS")) min_blocks = std::max(1, std::min(4, atoi(mb)));
   if (cmem) {

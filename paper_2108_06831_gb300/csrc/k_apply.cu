@@ -178,7 +178,16 @@ cudaError_t launch_forward(const tn_plan *p, const float2 *mats, long long mstri
       const size_t smem = p->jit_smem[i];
       cudaError_t e = cudaSuccess;
       long long work = (long long)p->batch << h.n_outer;
-      const long long grid = std::min<long long>(work, 1ll << 30);  // one tile per CTA
+      // One tile per CTA.  Where CTAs of less than half a warp (tiles of 6 and 7 qubits) would be more than 16 per
+      // SM, two or more each, up to 32 CTAs per SM: starting one takes longer than its tile (tiles of 64: 20
+      // qubits 384 us with one tile per CTA, 213 with four, 18 qubits 92, 65 with two; tiles of 128: 20 qubits
+      // 203, 130 with two, 18 qubits, 13 per SM, 54 either way; of 256, 16 threads: no difference).
+      long long grid = std::min<long long>(work, 1ll << 30);
+      if (threads < 16 && work > 16ll * num_sms()) {
+        long long tiles = 2;
+        while (work > tiles * 32 * num_sms()) tiles *= 2;
+        grid = (work + tiles - 1) / tiles;
+      }
       const float2 *m = mats;
       unsigned long long init = p->init;
       // per-call tables (parameterised, batch 1): this pass's entries into its constant table
