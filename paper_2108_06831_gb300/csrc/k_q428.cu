@@ -78,6 +78,8 @@ struct alignas(16) QPhase {
 };
 static_assert(sizeof(QPhase) == 32, "QPhase layout");
 constexpr int kQMaxPhases = 64;  // phases of one pass staged in shared memory
+// a gate mixes at most two bits, so every phase of a pass but the last holds at least two gates
+static_assert(kQReg == 4 && kQMaxPhases >= kQMaxOps / 2, "the ops of a pass bound its phases");
 
 struct alignas(16) QPass {
   int32_t T, n_outer, init;  // init: the first pass, whose tile is synthesised
@@ -659,7 +661,7 @@ Q428Plan *q428_build(const tn_circuit &c) {
     pd.phase_begin = (int)p->phases.size();
     pd.op_begin = (int)p->ops.size();
     pd.mat_begin = (int)p->mats.size();
-    while (k0 < k1 && (int)p->phases.size() - pd.phase_begin < kQMaxPhases) {
+    while (k0 < k1) {
       uint64_t R = 0;
       int k2 = k0;
       for (; k2 < k1; ++k2) {

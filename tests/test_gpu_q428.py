@@ -193,3 +193,22 @@ def test_pass_records_at_their_limits():
     gates += [C.Gate("U3", (3,), tuple(rng.uniform(0, 6, 3))) for _ in range(131)]
     gates += [C.Gate("U3", (int(4 * k % 9),), tuple(rng.uniform(0, 6, 3))) for k in range(300)]
     _assert_bit_exact(C.Circuit(n, gates, init_basis=300))
+
+
+def test_pass_of_64_phases():
+    """The most phases a pass can hold: 128 exchanges of which three in a row always mix six bits, after a pass of
+    128 one-qubit gates; states of one tile and of several."""
+    for n in (12, 13):
+        rng = np.random.default_rng(n)
+        def u3(k):
+            return C.Gate("U3", (k % n,), tuple(rng.uniform(0, 6, 3)))
+        pairs = [(n - 12 + 2 * j, n - 11 + 2 * j) for j in range(6)]
+        swaps = [C.Gate("SWAP", pairs[k % 6]) for k in range(128)]
+        phases, mixed = 1, set()
+        for g in swaps:
+            if len(mixed | set(g.qubits)) > 4:
+                phases, mixed = phases + 1, set()
+            mixed |= set(g.qubits)
+        assert phases == 64
+        first = [C.Gate("U3", (n - 1 - k % 12,), tuple(rng.uniform(0, 6, 3))) for k in range(128)]
+        _assert_bit_exact(C.Circuit(n, first + swaps + [u3(k) for k in range(n)], init_basis=1234))
