@@ -515,7 +515,7 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
     q->host_only = p->host_only;
     q->device = -1;
     q->T = T;
-    q->K = c->n <= 12 && T <= 12 ? kLeanReg : kLeanReg + 1;  // at most 1024 threads
+    q->K = c->n <= kLeanNarrow ? kLeanReg : kLeanReg + 1;
     q->is_lean = true;
     st = build_passes(c, o, q, err);
     if (st == TN_OK) {

@@ -26,17 +26,20 @@ constexpr int kMaxReg = 4;       // register qubits per thread and phase (2^4 am
 constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pass of the adjoint sweep
 // Small states: with 16 amplitudes a thread they give an SM too few warps to hide a pass's latency (every
 // gate is a chain of dependent instructions, every phase a barrier).  Below kLeanWarps warps per SM the
-// forward passes run from a plan of kLeanReg register qubits (four amplitudes a thread; one qubit more
-// for states of several tiles): more phases, but four times the warps and a quarter of the instructions
-// in each thread's way.  Below kLeanGates gates that mix amplitudes there is nothing to shorten.  From
-// kFuseMinQubitsParam qubits on a parameterised circuit's 4x4 blocks are read from shared memory by
+// forward passes run from a plan of kLeanReg register qubits (four amplitudes a thread), one more from
+// kLeanNarrow + 1 qubits on: more phases, but four times (twice) the warps and a quarter (half) of the
+// instructions in each thread's way.  Below kLeanGates gates that mix amplitudes there is nothing to shorten.
+// From kFuseMinQubitsParam qubits on a parameterised circuit's 4x4 blocks are read from shared memory by
 // twice the threads, which costs more than the warps gain (16 qubits, 8 sets: 47 against 55 us).
-// Measured: 9 qubits depth 6, one set 20.6 -> 10.4 us; 10 qubits depth 8, 128 sets 26.7 -> 14.4 us.
+// Measured with four, three and two register qubits: parameterised brickwork of depth 7, 9 qubits 20.4, 12.3
+// and 10.1 us, 10 qubits 20.6, 12.4 and 10.9, 11 qubits 22.7, 15.5 and 15.9, 12 qubits 28.8, 22.7 and 24.7,
+// 13 qubits 28.7, 26.7 and 28.9; hardware-efficient ansatz of 3 layers (weaker gates, a phase for every four
+// CNOTs), 10 qubits 13.9, 11.1 and 10.9, 11 qubits 14.4, 13.4 and 14.4, 12 qubits 18.5, 18.5 and 22.4.
 constexpr int kConstMinQubits = 19;  // parameterised circuits, batch 1: constant tables from this width on
 constexpr int kTargetSms = 152;      // GB300
 constexpr double kLeanWarps = 8.0;
 constexpr double kLeanGates = 24.0;
-constexpr int kLeanReg = 2;
+constexpr int kLeanReg = 2, kLeanNarrow = 11;
 
 // ---------------------------------------------------------------------------------------
 // Register-level operations of the fused gate-apply kernel.
