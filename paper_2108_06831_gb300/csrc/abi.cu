@@ -168,13 +168,13 @@ double lean_weight(const TnGate &g) {
   }
 }
 
-// Passes, tables and generated kernels of a state plan whose sizes (n, batch, T, K, ..) are set.  On
-// failure everything but p itself has been freed.
-tn_status build_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, std::string &err) {
+// Passes and workspace of a state plan whose sizes (n, batch, T, K, ..) are set, and the rewritten circuit
+// its forward passes run.
+tn_status plan_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, tn_circuit &fwd_circ, std::string &err) {
   // Precontracted blocks cost a per-call FP64 product when the circuit reads parameters; below
   // kFuseMinQubitsParam qubits that costs more than the smaller state saves in the passes.
   const bool fuse = !(o.flags & TN_PLAN_NO_FUSION) && (c->n_params == 0 || c->n >= kFuseMinQubitsParam);
-  const tn_circuit fwd_circ = push_phases(fuse ? fuse_pairs(*c, p->fused) : *c, p->fused);
+  fwd_circ = push_phases(fuse ? fuse_pairs(*c, p->fused) : *c, p->fused);
   for (const TnGate &g : fwd_circ.gates) p->n_fused += g.kind == KIND_F2 ? 1 : 0;
   tn_status st = build_pass_plan(fwd_circ, p->T, p->K, false, p->slots, p->fwd, err);
   // the adjoint sweep stages two tiles (psi, lambda): at most 2^11 amplitudes each
@@ -211,7 +211,11 @@ tn_status build_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, s
     off = align_up(off + (size_t)o.batch * kMaxRedPasses * 512 * sizeof(double));
   }
   p->ws_bytes = off;
+  return TN_OK;
+}
 
+// Tables and generated kernels of a planned state plan.  On failure everything but p itself has been freed.
+tn_status load_passes(const tn_circuit *c, const tn_plan_opts &o, tn_plan *p, const tn_circuit &fwd_circ) {
   if (p->host_only && getenv("TNQ_JIT_COMPILE_CHECK") && !(o.flags & TN_PLAN_NO_SPECIALIZE) && jit_supported(*p)) {
     // generate and compile the specialised kernels without loading them (no GPU needed)
     std::vector<int> kinds(p->fwd.ops.size());
@@ -492,18 +496,26 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
     *out = p;
     return TN_OK;
   }
+  tn_circuit fwd_circ;
+  tn_status st = plan_passes(c, o, p, fwd_circ, err);
+  if (st != TN_OK) {
+    delete p;
+    return st;
+  }
   // A plan of few warps (see kLeanWarps) runs its forward passes from a second, lean plan; the first
   // then only serves the batched executor's tables and needs no generated kernels.
   double mixing = 0.0;  // gates that mix amplitudes: permutations and diagonal gates are cheap either way
   for (const TnGate &g : c->gates) mixing += lean_weight(g);
   const double sms = p->host_only ? kTargetSms : num_sms();  // a host-only plan is the plan of a GB300
+  const double flops = std::ldexp(p->fwd.flops, -c->n);     // per amplitude
+  const bool deep = c->n_params > 0 ? c->n < kFuseMinQubitsParam
+                                    : flops >= (c->n < kLeanNarrow ? 0.0 : c->n == kLeanNarrow ? kLeanFlops : kLeanFlopsWide);
   const bool lean = o.target != TN_TARGET_EXPECTATION && !(o.flags & TN_PLAN_NO_SPECIALIZE) &&
-                    T >= kLowBits + 2 && c->n < kBatchDirectMinQubits && mixing >= kLeanGates &&
-                    (c->n_params == 0 || c->n < kFuseMinQubitsParam) &&
+                    T >= kLowBits + 2 && c->n < kBatchDirectMinQubits && mixing >= kLeanGates && deep &&
                     std::ldexp((double)o.batch, c->n - 9) < kLeanWarps * sms;
   tn_plan_opts o_main = o;
   if (lean) o_main.flags |= TN_PLAN_NO_SPECIALIZE;
-  tn_status st = build_passes(c, o_main, p, err);
+  st = load_passes(c, o_main, p, fwd_circ);
   if (st == TN_OK && lean) {
     tn_plan *q = new tn_plan();
     q->n = p->n;
@@ -517,14 +529,16 @@ tn_status tn_plan_contraction(const tn_circuit *c, const tn_plan_opts *opts, tn_
     q->T = T;
     q->K = c->n <= kLeanNarrow ? kLeanReg : kLeanReg + 1;
     q->is_lean = true;
-    st = build_passes(c, o, q, err);
+    tn_circuit lean_circ;
+    st = plan_passes(c, o, q, lean_circ, err);
+    if (st == TN_OK) st = load_passes(c, o, q, lean_circ);
     if (st == TN_OK) {
       p->lean = q;
       p->ws_bytes = std::max(p->ws_bytes, q->ws_bytes);
     } else {
       delete q;
       jit_release(*p);
-      free_plan_device(p);
+      if (!p->host_only) free_plan_device(p);
     }
   }
   if (st != TN_OK) {

@@ -515,6 +515,12 @@ std::string gen_pass(const tn_plan &p, int pi, const std::vector<int> &op_kind, 
   // blocks; with them three, two when their entries are staged in shared memory (18 qubits, one set: 41 us
   // with two, 66 with three; 24 qubits from constant memory 1195, 1060 and 1122 us with two, three and four)
   int min_blocks = !blocks ? 4 : cmem ? 3 : 2;
+  // At most two where no SM has more CTAs than that to run (but not for the widths that batches run beside
+  // other circuits' CTAs): 96 small states of 12-18 qubits took on average 2.5 and 7% longer with three and four
+  // than with two, and no less with one; 18-qubit ansatz of 10 layers, five sets 150 and 140 us.
+  const long long ctas = (((long long)p.batch << pd.n_outer) + kTargetSms - 1) / kTargetSms;  // per SM
+  if (p.n < kBatchDirectMinQubits || p.batch > 1)
+    min_blocks = (int)std::min<long long>(min_blocks, std::max<long long>(2, ctas));
   // These are CTAs of 256 threads: tiles of 13 qubits, 512 threads, would be left 32 or 42 registers and spill
   // (20-qubit brickwork 56 us with three, 27 with one; 20-qubit energies of two sets 342 with four, 94 with two)
   if (NTHR > 256) min_blocks = std::max(1, min_blocks * 256 / NTHR);

@@ -120,7 +120,6 @@ cudaError_t launch_cgemm(int precision, long long batch, long long M, long long 
 
 // Persistent batched executor.  Circuits of at least kBatchDirectMinQubits qubits whose plans carry
 // generated pass kernels run those kernels on side streams instead (at least 128 tiles per pass).
-constexpr int kBatchDirectMinQubits = 19;
 tn_status batch_build(const tn_plan *const *plans, int n, tn_batch **out);
 // params: every parameterised circuit's parameters back to back (NULL when none has any).
 cudaError_t batch_run(const tn_batch *b, const double *params, float2 *states, void *ws, cudaStream_t s);

@@ -28,18 +28,27 @@ constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pas
 // gate is a chain of dependent instructions, every phase a barrier).  Below kLeanWarps warps per SM the
 // forward passes run from a plan of kLeanReg register qubits (four amplitudes a thread), one more from
 // kLeanNarrow + 1 qubits on: more phases, but four times (twice) the warps and a quarter (half) of the
-// instructions in each thread's way.  Below kLeanGates gates that mix amplitudes there is nothing to shorten.
+// instructions in each thread's way.  All times are of calls replayed from a graph unless they say otherwise.
+//   kLeanWarps: 9-qubit brickwork of depth 6 with four and two register qubits, 6 warps per SM 26.4 and 20.9 us,
+//   8 35.7 and 32.2, 16 55.6 and 51.6; ansatz of 3 layers 27.6 and 27.5, 30.5 and 31.8, 53.2 and 55.4.
+//   kLeanGates: fewer gates that mix amplitudes than this gain nothing in eager calls, which the launches bound
+//   (8-qubit brickwork of depth 2, 16 gates: 10 us either way, though 8.5 and 6.3 from a graph).
+//   kLeanNarrow, four, three and two register qubits in eager calls: parameterised brickwork of depth 7, 9 qubits
+//   20.4, 12.3 and 10.1 us, 11 qubits 22.7, 15.5 and 15.9, 12 qubits 28.8, 22.7 and 24.7; ansatz of 3 layers,
+//   10 qubits 13.9, 11.1 and 10.9, 11 qubits 14.4, 13.4 and 14.4, 12 qubits 18.5, 18.5 and 22.4.
+//   kLeanFlops, kLeanFlopsWide: below this many FP32 operations per amplitude fixed angles lose by the added
+//   phases, at kLeanNarrow qubits (Fig. 3.1 circuits of 1 layer, 299: 3.8 and 4.3 us, of 2, 466: 6.1 and 5.3) and
+//   above (14 qubits: depth 5 in single gates, 373: 12.6 and 13.3, depth 7, 605: 15.3 and 16.7, depth 10, 1007:
+//   27.6 and 23.5; 18 qubits: Fig. 3.1 of 2 layers, 386: 15.1 and 16.1, of 4, 894: 29.7 and 25.0).
 // From kFuseMinQubitsParam qubits on a parameterised circuit's 4x4 blocks are read from shared memory by
 // twice the threads, which costs more than the warps gain (16 qubits, 8 sets: 47 against 55 us).
-// Measured with four, three and two register qubits: parameterised brickwork of depth 7, 9 qubits 20.4, 12.3
-// and 10.1 us, 10 qubits 20.6, 12.4 and 10.9, 11 qubits 22.7, 15.5 and 15.9, 12 qubits 28.8, 22.7 and 24.7,
-// 13 qubits 28.7, 26.7 and 28.9; hardware-efficient ansatz of 3 layers (weaker gates, a phase for every four
-// CNOTs), 10 qubits 13.9, 11.1 and 10.9, 11 qubits 14.4, 13.4 and 14.4, 12 qubits 18.5, 18.5 and 22.4.
 constexpr int kConstMinQubits = 19;  // parameterised circuits, batch 1: constant tables from this width on
 constexpr int kTargetSms = 152;      // GB300
+constexpr int kBatchDirectMinQubits = 19;  // widths from which a batch runs a circuit's own kernels
 constexpr double kLeanWarps = 8.0;
 constexpr double kLeanGates = 24.0;
 constexpr int kLeanReg = 2, kLeanNarrow = 11;
+constexpr double kLeanFlops = 400.0, kLeanFlopsWide = 700.0;
 
 // ---------------------------------------------------------------------------------------
 // Register-level operations of the fused gate-apply kernel.

@@ -301,10 +301,11 @@ def test_small_plans_compile_without_a_device(tmp_path, monkeypatch):
 
     def reg_qubits(circ, **kw):
         return tn.Plan(tn.CircuitHandle(circ), host_only=True, **kw).stats()["reg_qubits"]
-    nine, fixed = C.brickwork(9, 6, 5, parameterized=True)[0], C.brickwork(14, 4, 5)[0]
+    nine, fixed = C.brickwork(9, 6, 5, parameterized=True)[0], C.brickwork(14, 16, 5)[0]
     assert reg_qubits(nine) == 2 and reg_qubits(C.qft(10, 3), target=tn.TARGET_AMPLITUDES) == 4
     assert reg_qubits(nine, target=tn.TARGET_AMPLITUDES) == 2 and reg_qubits(fixed) == 3
     assert [reg_qubits(C.hea(n, 3)) for n in (6, 8, 11, 12, 13)] == [4, 2, 2, 3, 3]
+    assert [reg_qubits(C.brickwork(n, 3, 5)[0]) for n in (10, 11, 12, 18)] == [2, 4, 4, 4]  # too few operations
     assert reg_qubits(nine, batch=1215) == 2 and reg_qubits(nine, batch=1216) == 4  # 8 warps on each of 152 SMs
     assert reg_qubits(nine, specialize=False) == 4 and reg_qubits(nine, target=tn.TARGET_EXPECTATION) == 4
     srcs = [f.read_text() for f in dump.glob("*.cu")]
