@@ -515,8 +515,9 @@ bool is_zero(const int32_t *e) { return e[0] == 0 && e[1] == 0; }
 struct QForm {
   int type;
   bool mix_a, mix_b, heavy;
-  std::vector<int32_t> mat;
-  uint8_t ones = 0;
+  uint8_t ones;
+  int n_mat;
+  int32_t mat[32];
 };
 QForm form_of(const Q428Gate &g) {
   QForm f{};
@@ -529,17 +530,17 @@ QForm form_of(const Q428Gate &g) {
   if (diag) {
     // entry 2 bit(a) + bit(b); a one-qubit gate has a = b (entries 0 and 3)
     f.type = Q_DIAG;
-    f.mat.assign(8, 0);
+    f.n_mat = 8;
     for (int v = 0; v < 4; ++v) {
       const int32_t *d = dim == 4 ? e(v, v) : e(v >> 1, v >> 1);
       f.mat[2 * v] = d[0];
       f.mat[2 * v + 1] = d[1];
       if (is_one(d)) f.ones |= (uint8_t)(1 << v);
     }
-    const int32_t *last = f.mat.data() + 6;
-    if (last[0] == -(1 << 28) && last[1] == 0 && (dim == 4 ? f.ones == 7 : is_one(f.mat.data()))) {
+    const int32_t *last = f.mat + 6;
+    if (last[0] == -(1 << 28) && last[1] == 0 && (dim == 4 ? f.ones == 7 : is_one(f.mat))) {
       f.type = Q_NEG;
-      f.mat.clear();
+      f.n_mat = 0;
     }
     return f;
   }
@@ -561,10 +562,13 @@ QForm form_of(const Q428Gate &g) {
     if (f.type == Q_G1 || f.type == Q_V1) {
       for (int k = 0; k < 4; ++k) {
         const int32_t ur = u[2 * k], ui = u[2 * k + 1];
-        f.mat.insert(f.mat.end(), {ur, -(ur + ui), ui - ur});
+        f.mat[f.n_mat++] = ur;
+        f.mat[f.n_mat++] = -(ur + ui);
+        f.mat[f.n_mat++] = ui - ur;
       }
     } else {
-      f.mat.assign(u, u + 8);
+      std::copy(u, u + 8, f.mat);
+      f.n_mat = 8;
     }
     return f;
   }
@@ -582,7 +586,10 @@ QForm form_of(const Q428Gate &g) {
   }
   f.mix_a = f.mix_b = f.heavy = true;
   f.type = perm_is(swap) ? Q_SWAP : Q_G2;
-  if (f.type == Q_G2) f.mat.assign(g.u, g.u + 32);
+  if (f.type == Q_G2) {
+    std::copy(g.u, g.u + 32, f.mat);
+    f.n_mat = 32;
+  }
   return f;
 }
 
@@ -607,6 +614,7 @@ int32_t q428_quantize(double x) {
 
 Q428Plan *q428_build(const tn_circuit &c) {
   Q428Plan *p = new Q428Plan();
+  p->gates.reserve(c.gates.size());
   for (const TnGate &g : c.gates) {
     double m[32];
     const int dim = gate_matrix(g.kind, FORM_U, g.angle, g.mat, m);
@@ -620,8 +628,11 @@ Q428Plan *q428_build(const tn_circuit &c) {
   const int n = c.n, G = (int)p->gates.size();
   if (n < kQMinQubits || G == 0) return p;
   const int T = std::min(n, kQTile);
-  std::vector<QForm> forms;
-  for (const Q428Gate &g : p->gates) forms.push_back(form_of(g));
+  std::vector<QForm> forms((size_t)G);
+  size_t entries = 0;
+  for (int k = 0; k < G; ++k) entries += (size_t)(forms[(size_t)k] = form_of(p->gates[(size_t)k])).n_mat;
+  p->ops.reserve((size_t)G);
+  p->mats.reserve(entries);
   auto mixed = [&](int k) {  // state bits gate k mixes
     uint64_t b = 0;
     if (forms[(size_t)k].mix_a) b |= 1ull << p->gates[(size_t)k].pos[0];
@@ -637,7 +648,7 @@ Q428Plan *q428_build(const tn_circuit &c) {
     int k1 = k0, n_mat = 0;
     for (; k1 < G && k1 - k0 < kQMaxOps; ++k1) {
       const uint64_t U = S | mixed(k1);
-      const int nm = (int)forms[(size_t)k1].mat.size();
+      const int nm = forms[(size_t)k1].n_mat;
       if (__builtin_popcountll(U) > T || n_mat + nm > kQMaxMat) break;
       S = U;
       n_mat += nm;
@@ -682,21 +693,19 @@ Q428Plan *q428_build(const tn_circuit &c) {
         }
       // thread bits: the first five (lanes) cover the residues mod 4 where they can, so a warp's
       // shared-memory accesses fall in distinct banks under the tile's swizzle
-      std::vector<int> rest;
+      int rest[kQTile], n_rest = 0, t = 0;
+      bool used[kQTile] = {};
       for (int b = 0; b < n; ++b)
-        if (((S >> b) & 1) && !((R >> b) & 1)) rest.push_back(tile_of[b]);
-      std::vector<int> order;
-      std::vector<char> used(rest.size(), 0);
+        if (((S >> b) & 1) && !((R >> b) & 1)) rest[n_rest++] = tile_of[b];
       for (int res = 0; res < 4; ++res)
-        for (size_t i = 0; i < rest.size(); ++i)
+        for (int i = 0; i < n_rest; ++i)
           if (!used[i] && (rest[i] & 3) == res) {
-            order.push_back(rest[i]);
-            used[i] = 1;
+            ph.thr_pos[t++] = (uint8_t)rest[i];
+            used[i] = true;
             break;
           }
-      for (size_t i = 0; i < rest.size(); ++i)
-        if (!used[i]) order.push_back(rest[i]);
-      for (size_t i = 0; i < order.size(); ++i) ph.thr_pos[i] = (uint8_t)order[i];
+      for (int i = 0; i < n_rest; ++i)
+        if (!used[i]) ph.thr_pos[t++] = (uint8_t)rest[i];
       auto source = [&](int bit, uint8_t &kind, uint8_t &pos) {
         if (reg_of[bit] >= 0) kind = SRC_REG, pos = (uint8_t)reg_of[bit];
         else if (tile_of[bit] >= 0) kind = SRC_TILE, pos = (uint8_t)tile_of[bit];
@@ -715,7 +724,7 @@ Q428Plan *q428_build(const tn_circuit &c) {
         if (f.type == Q_X1 && g.nq == 1) op.a_kind = kAlways;
         pd.heavy |= f.heavy ? 1 : 0;
         op.mat = (int)p->mats.size() - pd.mat_begin;
-        p->mats.insert(p->mats.end(), f.mat.begin(), f.mat.end());
+        p->mats.insert(p->mats.end(), f.mat, f.mat + f.n_mat);
         p->ops.push_back(op);
       }
       ph.op_end = (int)p->ops.size();
