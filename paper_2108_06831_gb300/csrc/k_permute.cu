@@ -17,6 +17,7 @@
 // Every mbarrier wait is bounded: on expiry the kernel records TN_ERR_TIMEOUT in the
 // device status word and returns.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "apply_common.cuh"
@@ -33,12 +34,13 @@ constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of every mbarrie
 
 constexpr int kPermLo = 6;          // low bits: runs of 64 elements = 512 bytes
 constexpr int kPermMaxRowBits = 6;  // at most 64 rows per tile
+constexpr int kPermMinRowBits = 3;  // a row per warp
 
 struct PermParams {
   int n, lo, e, r, n_outer;       // r = row bits of a tile (e extra + r - e passive)
   int row_stride;                 // shared-memory row stride (elements, multiple of 2)
   uint8_t extra_in[8];            // input bit of extra (row) bit q
-  uint8_t col_from_k[8];          // for output low bit j: input bit o_in[j]
+  int lane_bit[kPermLo];          // output low bit j's offset within a stage: a column bit's or a row's
   uint8_t m_in[8];                // input low bits not feeding output low bits (run-index bits)
   uint8_t m_out[8];               // their output bit positions
   uint8_t pas_in[8], pas_out[8];  // passive row bits: input and output bit positions
@@ -109,16 +111,10 @@ __global__ void __launch_bounds__(kPermThreads) k_permute(PermParams P, long lon
 
   if (threadIdx.x < runlen) {
     const int k = threadIdx.x;
-    int row = 0, col = 0;
-    for (int j = 0; j < P.lo; ++j) {
-      const int ib = P.col_from_k[j];
-      const int v = (k >> j) & 1;
-      if (ib < P.lo) col |= v << ib;
-      else
-        for (int q = 0; q < P.e; ++q)
-          if (P.extra_in[q] == ib) row |= v << q;
-    }
-    lane_off[k] = row * P.row_stride + col;
+    int at = 0;
+#pragma unroll
+    for (int j = 0; j < kPermLo; ++j) at += ((k >> j) & 1) ? P.lane_bit[j] : 0;
+    lane_off[k] = at;
   }
   if (threadIdx.x < rows) {
     // row m of the tile: bits [0, e) extra, bits [e, r) passive.  As a write index, the low
@@ -241,12 +237,13 @@ cudaError_t launch_permute(int n, const int32_t *perm, long long batch, const fl
   }
   const int lo = kPermLo;
   P.lo = lo;
+  P.row_stride = (1 << lo) + 2;
   bool in_S[64] = {false};
   for (int b = 0; b < lo; ++b) in_S[b] = true;
   int e = 0;
   for (int j = 0; j < lo; ++j) {
     const int ib = in_of_out[j];
-    P.col_from_k[j] = (uint8_t)ib;
+    P.lane_bit[j] = ib < lo ? 1 << ib : P.row_stride << e;
     if (ib >= lo) {
       in_S[ib] = true;
       P.extra_in[e++] = (uint8_t)ib;
@@ -265,12 +262,16 @@ cudaError_t launch_permute(int n, const int32_t *perm, long long batch, const fl
       ++mq;
     }
   }
-  // passive row bits (lowest remaining input bits) fill the tile up to 64 rows; the rest
-  // index tiles
+  // passive row bits (lowest remaining input bits) fill the tile up to 64 rows, fewer where the tiles would not
+  // give every SM two (replayed from a graph, 18 legs: 5.7-6.0 us with 64 rows, 4.2-4.8 with fewer; 12 legs 5.6 and
+  // 3.5); the rest index
+  // tiles
+  int max_r = kPermMaxRowBits;
+  while (max_r > kPermMinRowBits && std::ldexp((double)batch, n - lo - max_r) < 2.0 * num_sms()) --max_r;
   int no = 0;
   for (int b = 0; b < n; ++b)
     if (!in_S[b]) {
-      if (P.r < kPermMaxRowBits) {
+      if (P.r < max_r) {
         P.pas_in[P.r - e] = (uint8_t)b;
         P.pas_out[P.r - e] = (uint8_t)out_of_in[b];
         ++P.r;
@@ -281,7 +282,6 @@ cudaError_t launch_permute(int n, const int32_t *perm, long long batch, const fl
       ++no;
     }
   P.n_outer = no;
-  P.row_stride = (1 << lo) + 2;
   const size_t smem = (size_t)kPermStages * (1 << P.r) * P.row_stride * sizeof(float2);
   cudaError_t err = ensure_smem(reinterpret_cast<const void *>(k_permute), smem);
   if (err != cudaSuccess) return err;
