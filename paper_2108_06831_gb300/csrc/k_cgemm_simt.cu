@@ -230,9 +230,14 @@ __global__ void __launch_bounds__(kThreads, MINB) k_cgemm_fp32(long long M, long
 // memory (cache-resident at this size) and stores through the output map, without tile
 // staging.  The accumulation over k is the tiled kernel's (same order, same fused
 // multiply-adds), so both give the same bits.
+// The map goes bit by bit where there are few elements and so few bits (a run's shifts and loads take longer
+// than two bits': 3 x 3 grid of depth 6, replayed from a graph, 13.0 us, 13.9 with runs), in runs where there are many.
+__device__ __forceinline__ long long stored(const MapRuns &om, long long f) { return map_runs(om, f); }
+__device__ __forceinline__ long long stored(const OutMap &om, long long f) { return om.identity ? f : map_bits(om, f, 0); }
+template <class Map>
 __global__ void __launch_bounds__(256) k_cgemm_small(long long M, long long N, long long K, long long total,
                                                      const float2 *__restrict__ A, const float2 *__restrict__ B,
-                                                     float2 *__restrict__ C, const __grid_constant__ MapRuns om) {
+                                                     float2 *__restrict__ C, const __grid_constant__ Map om) {
   pdl_wait();
   pdl_trigger();
   for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < total;
@@ -249,10 +254,11 @@ __global__ void __launch_bounds__(256) k_cgemm_small(long long M, long long N, l
       acc.y = fmaf(x.x, y.y, acc.y);
       acc.y = fmaf(x.y, y.x, acc.y);
     }
-    C[map_runs(om, f)] = acc;
+    C[stored(om, f)] = acc;
   }
 }
 constexpr long long kSmallWork = 1ll << 18;
+constexpr long long kFewElements = 1ll << 14;
 
 // Sum of the split-K partials (in split order) of every output element, stored through the
 // output map: C[map(f)] = sum_s P[s][f], f the natural index (b M + m) N + n.
@@ -424,7 +430,9 @@ cudaError_t launch_cgemm_fp32(long long batch, long long M, long long N, long lo
   // 13.1, none 22.4)
   if (K <= 64 && ((double)total * (double)K <= (double)kSmallWork || N <= 4)) {
     const long long blocks = std::min<long long>((total + 255) / 256, (long long)num_sms() * 16);
-    return launch_pdl(k_cgemm_small, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, runs_of(m));
+    if (total <= kFewElements)
+      return launch_pdl(k_cgemm_small<OutMap>, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, m);
+    return launch_pdl(k_cgemm_small<MapRuns>, dim3((unsigned)blocks), dim3(256), 0, s, M, N, K, total, A, B, C, runs_of(m));
   }
   if (P != nullptr) {  // few tiles: the short ones
     if (N <= 8) return launch_tiles<true, 32, 8, 2, 1, 8>(batch, M, N, K, A, B, C, P, m, s);
