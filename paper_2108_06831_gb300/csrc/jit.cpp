@@ -478,7 +478,7 @@ bool jit_const_mats(const tn_plan &p) {
   if (const char *e = getenv("TNQ_JIT_CONST"))
     if (atoi(e) == 0) return false;
   // per-call tables of smaller states are staged in shared memory: the copies into the constant tables, one
-  // before each pass, cost more than they save (16 qubits depth 10: 47 us with them, 37 without; 22: 159, 170)
+  // before each pass, cost more than they save (times at kConstMinQubits)
   return !p.param_dependent || (p.batch == 1 && p.n >= kConstMinQubits);
 }
 

@@ -22,7 +22,10 @@ namespace tnq {
 // slot or member, and now: 10-qubit brickwork of depth 8, 16 sets 14.4 and 12.4 us; 16 qubits, depth 10,
 // one set 37 and 33 us; 22 qubits 159 and 155 us.
 constexpr long long kFusedPerThread = 1024;  // fused blocks x batch from which each takes one thread
-constexpr long long kSpreadSlots = 4096;     // other slots x batch up to which each takes four threads
+// Other slots x batch up to which each takes four threads: whole calls with one thread per slot and with four,
+// 10 qubits, replayed from a graph: U3 slots 2560 12.2 and 11.2 us, 5120 12.2 and 11.5, 10240 12.4 and 13.6;
+// slots of one angle 1920 10.1 either way, 3840 9.8 and 10.7.
+constexpr long long kSpreadSlots = 4096;
 
 // One regular slot (one gate's matrix) for one batch element; prow: its parameters (may be NULL).
 __device__ void materialize_one(const MatSlot &s, const double *prow, float2 *table) {

@@ -16,14 +16,14 @@
 // registers.  Diagonal gates and a CNOT's control mix nothing and read any bit, of the register
 // index, the thread or the tile.
 //
-// Bound: the widening 32-bit multiplier (the heavy half of the FMA pipe, about 32 products per SM
-// and clock) and the latency in front of it.  A U3 takes 11 products per amplitude pair (Gauss); a
-// pass's memory traffic (16 bytes per amplitude) is shared by about 16 gates and hides behind the
-// arithmetic of the SM's other CTAs.  24-qubit brickwork of depth 20 (480 U3, 231 CZ in 45 passes):
-// 11.2 ms, 34.4 ms with one launch per gate (711 launches, each at 82% of the copy bandwidth).
-// Warps count for more than registers: 2, 3 and 4 CTAs of 256 threads per SM (128, 80 and 64
-// registers) measured 18.9, 13.0 and 11.3 ms; 2^11-amplitude tiles 13.4 ms (more passes), 8
-// amplitudes a thread 13.6 ms (more phases).
+// Bound: the widening 32-bit multiplier (the heavy half of the FMA pipe: 21.7 multiply-adds of 32 x 32 bits
+// onto 64 per SM and clock, 6.82e12 a second, measured with 16 independent chains per thread) and the latency in
+// front of it.  A U3 takes 11 products per amplitude pair (Gauss); a pass's memory traffic (16 bytes per
+// amplitude) is shared by about 14 gates and hides behind the arithmetic of the SM's other CTAs.  24-qubit
+// brickwork of depth 20 (480 U3, 230 CZ in 50 passes, 4.4e10 products: 6.5 ms at that rate): 11.2 ms, 58% of the
+// rate; 34.4 ms with one launch per gate (711 launches, each at 82% of the copy bandwidth).
+// Warps count for more than registers: 2, 3 and 4 CTAs of 256 threads per SM (128, 80 and 64 registers) measured
+// 18.9, 13.0 and 11.3 ms; 2^11-amplitude tiles 13.4 ms (more passes), 8 amplitudes a thread 13.6 (more phases).
 #include <algorithm>
 #include <climits>
 #include <cmath>

@@ -42,7 +42,12 @@ constexpr int kMaxGradSlots = 256;  // parameter derivatives accumulated per pas
 //   27.6 and 23.5; 18 qubits: Fig. 3.1 of 2 layers, 386: 15.1 and 16.1, of 4, 894: 29.7 and 25.0).
 // From kFuseMinQubitsParam qubits on a parameterised circuit's 4x4 blocks are read from shared memory by
 // twice the threads, which costs more than the warps gain (16 qubits, 8 sets: 47 against 55 us).
-constexpr int kConstMinQubits = 19;  // parameterised circuits, batch 1: constant tables from this width on
+// Parameterised circuits, batch 1: constant tables (copied before each pass) from this width on, staged in shared
+// memory below.  Replayed from a graph, staged and constant: brickwork of depth 7, 18 qubits 27.0 and 30.5 us, 19
+// 29.0 and 31.4, 20 41.1 and 40.2, 22 114 and 101; ansatz of 10 layers, 18 qubits 74 and 83, 20 126 and 139, 22 337
+// and 325.  From 19 on batches run these kernels on several streams at once, where constant tables leave the
+// shared memory to the others.
+constexpr int kConstMinQubits = 19;
 constexpr int kTargetSms = 152;      // GB300
 constexpr int kBatchDirectMinQubits = 19;  // widths from which a batch runs a circuit's own kernels
 constexpr double kLeanWarps = 8.0;
