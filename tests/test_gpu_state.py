@@ -316,3 +316,16 @@ def test_diagonal_gates_leave_what_their_condition_excludes(n, tile):
         ref = simulate_state(C.Circuit(n, h + phases)).reshape(1 << q, 2, -1)
         assert np.all(np.isposinf(got[:, 0].real)) and np.all(got[:, 0].imag == 0), q
         assert rel_l2(got[:, 1], ref[:, 1]) <= STATE_TOL, q
+
+
+@pytest.mark.parametrize("n,tile,batch", [(18, 6, 1), (20, 7, 1), (19, 7, 1), (12, 6, 77), (17, 6, 2)])
+def test_small_tiles_share_ctas(n, tile, batch):
+    """CTAs of a few threads that take several tiles each: shares that divide the tiles and that do not, several
+    batch elements (whose tables change within a CTA's share)."""
+    from oracle.statevector import simulate_state
+    c, _ = C.brickwork(n, 3, 60 + n, parameterized=batch > 1)
+    c.init_basis = (n * 7919) % (1 << n)
+    params = np.random.default_rng(n).uniform(0, 2 * np.pi, size=(batch, c.n_params)) if batch > 1 else None
+    got = gpu_state(c, params, batch=batch, tile=tile)
+    for b in sorted({0, batch // 2, batch - 1}):
+        assert rel_l2(got[b], simulate_state(c, None if params is None else params[b])) <= STATE_TOL
